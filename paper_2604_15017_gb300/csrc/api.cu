@@ -817,8 +817,7 @@ int us_scene_upload(us_ctx* ctx, const us_scene_desc* d, uint64_t* scene_id) {
       (s = up(o.tri_e2, &sc.dev.tri_e2)) || (s = up(o.scat, &sc.dev.scat)) ||
       (s = up(o.nodes_t, &sc.dev.nodes_t)) || (s = up(o.prims_t, &sc.dev.prims_t)) ||
       (s = up(o.nodes4, &sc.dev.nodes4)) ||
-      (s = up(o.cell_sph, &sc.dev.cell_sph)) || (s = up(o.cell2, &sc.dev.cell2)) ||
-      (s = up_bytes(o.cell.data(), o.cell.size() * sizeof(uint32_t), reinterpret_cast<const void**>(&sc.dev.cell)))) {
+      (s = up(o.cell_rec, &sc.dev.cell_rec))) {
     for (void* p : sc.allocs) cudaFree(p);
     ctx->used -= sc.bytes;
     return s;

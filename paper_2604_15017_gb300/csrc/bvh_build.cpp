@@ -375,11 +375,11 @@ static void build_tri_bvh(const HostSceneIn& in, std::vector<float>& nodes_out, 
 const double GRID_CELLS_PER_SPHERE = 2.0;
 const double GRID_MAX_CELLS = 16.0 * 1024 * 1024;
 const double GRID_PAD = 1e-2;
+const float REC_EMPTY = NAN;  // centre of an empty entry: every test of it fails
 
 static void build_scatter_grid(const HostSceneIn& in, HostSceneOut& out) {
   const int ns = in.n_scat;
-  out.cell.clear();
-  out.cell_sph.clear();
+  out.cell_rec.clear();
   if (ns == 0) {
     out.gn[0] = out.gn[1] = out.gn[2] = 0;
     return;
@@ -417,7 +417,7 @@ static void build_scatter_grid(const HostSceneIn& in, HostSceneOut& out) {
       c1 = std::max(0, std::min(n[a] - 1, (int)std::floor((c + rs + pad - out.glo[a]) / out.gh)));
     };
     const size_t n_cells = (size_t)n[0] * n[1] * n[2];
-    std::vector<uint32_t> count(n_cells, 0), first(n_cells, 0);
+    std::vector<uint32_t> count(n_cells, 0);
     auto for_cells = [&](int j, auto&& fn) {
       int r0[3], r1[3];
       for (int a = 0; a < 3; ++a) cell_range(in.scat_pos[3 * (size_t)j + a], a, r0[a], r1[a]);
@@ -426,41 +426,39 @@ static void build_scatter_grid(const HostSceneIn& in, HostSceneOut& out) {
           for (int x = r0[0]; x <= r1[0]; ++x) fn(((uint32_t)z * n[1] + y) * n[0] + x);
     };
     for (int j = 0; j < ns; ++j) for_cells(j, [&](uint32_t c) { count[c]++; });
-    uint64_t acc = 0;
+    uint64_t acc = 0, n_recs = n_cells;
     uint32_t most = 0;
     for (size_t c = 0; c < n_cells; ++c) {
-      first[c] = (uint32_t)acc;
       acc += count[c];
       most = std::max(most, count[c]);
+      if (count[c] > 2) n_recs += (count[c] - 1) / 2;
     }
     if (most > 255 || acc >= (1u << 24)) continue;
-    out.cell.resize(n_cells);
-    for (size_t c = 0; c < n_cells; ++c) out.cell[c] = first[c] << 8 | count[c];
-    out.cell_sph.assign(4 * (size_t)acc, 0.0f);
+    // chain records of crowded cells follow the cells' own; entries fill a chain in order
+    out.cell_rec.assign(8 * n_recs, REC_EMPTY);
+    for (size_t r = 0; r < n_recs; ++r) out.cell_rec[8 * r + 3] = out.cell_rec[8 * r + 7] = 0.0f;
+    std::vector<uint32_t> tail(n_cells), filled(n_cells, 0);
+    for (size_t c = 0; c < n_cells; ++c) tail[c] = (uint32_t)c;
+    uint32_t n_chain = 0;  // at most acc / 2 < 2^23
     for (int j = 0; j < ns; ++j)
       for_cells(j, [&](uint32_t c) {
-        float* e = &out.cell_sph[4 * (size_t)first[c]++];
+        if (filled[c] == 2) {
+          float* r = &out.cell_rec[8 * (size_t)tail[c]];
+          uint32_t w0, w1;
+          std::memcpy(&w0, &r[3], 4);
+          std::memcpy(&w1, &r[7], 4);
+          ++n_chain;
+          r[3] = bits_f(w0 | (n_chain >> 12) << 20);
+          r[7] = bits_f(w1 | (n_chain & 0xFFFu) << 20);
+          tail[c] = (uint32_t)n_cells + n_chain - 1;
+          filled[c] = 0;
+        }
+        float* e = &out.cell_rec[8 * (size_t)tail[c] + 4 * filled[c]++];
         e[0] = in.scat_pos[3 * (size_t)j];
         e[1] = in.scat_pos[3 * (size_t)j + 1];
         e[2] = in.scat_pos[3 * (size_t)j + 2];
-        e[3] = bits_f((3u << 20) | (uint32_t)j);
+        e[3] = bits_f((uint32_t)j);
       });
-    // the first two entries of every cell inline, so that a ray reads one 32-byte record per
-    // cell: code 0 marks an empty slot, bit 31 of the second code that the cell holds more
-    out.cell2.assign(8 * n_cells, 0.0f);
-    for (size_t c = 0; c < n_cells; ++c) {
-      const uint32_t f0 = out.cell[c] >> 8, k = out.cell[c] & 0xFFu;
-      for (uint32_t slot = 0; slot < 2 && slot < k; ++slot) {
-        const float* e = &out.cell_sph[4 * (size_t)(f0 + slot)];
-        float* o = &out.cell2[8 * c + 4 * slot];
-        o[0] = e[0];
-        o[1] = e[1];
-        o[2] = e[2];
-        uint32_t code;
-        std::memcpy(&code, &e[3], 4);
-        o[3] = bits_f(code | (slot == 1 && k > 2 ? 0x80000000u : 0u));
-      }
-    }
     return;
   }
   // unreachable for scenes the upload accepts (< 2^20 spheres): an empty grid would lose hits

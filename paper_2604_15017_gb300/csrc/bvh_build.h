@@ -23,14 +23,14 @@ struct HostSceneOut {
   int n_nodes4 = 0, depth4 = 0;    // the same tree collapsed to 4-wide nodes (same leaves)
   std::vector<float> nodes4;       // 32 floats per node
   // uniform grid over the scatterer spheres: cell (x, y, z) covers glo + h [x, x+1) x [y, y+1) x
-  // [z, z+1).  cell[(z * gn[1] + y) * gn[0] + x] = first << 8 | count names the (centre, code)
-  // entries of every sphere whose (slightly inflated) bounding box overlaps the cell:
-  // cell_sph[first .. first + count)
+  // [z, z+1) and lists every sphere whose (slightly inflated) bounding box overlaps it, in
+  // records of two 16-byte entries (centre, sphere id | part of `next` << 20).  Record
+  // (z * gn[1] + y) * gn[0] + x is the cell's first; `next`, 24 bits (the high 12 in the first
+  // entry, the low 12 in the second), names the record that follows in a crowded cell, record
+  // (number of cells) + next - 1, or is 0.  An empty entry's centre is NaN.
   float glo[3] = {0, 0, 0}, gh = 1.0f;
   int gn[3] = {0, 0, 0};
-  std::vector<uint32_t> cell;
-  std::vector<float> cell_sph;  // 4 floats per entry
-  std::vector<float> cell2;     // per cell its first two entries (8 floats); see build_scatter_grid
+  std::vector<float> cell_rec;  // 8 floats per record
   std::vector<float> tri_nrm;  // 4 per triangle
   std::vector<float> tri_v0;   // 4 per triangle
   std::vector<float> tri_e1;   // 4 per triangle: (v1 - v0, |(v1 - v0) x (v2 - v0)|)

@@ -58,12 +58,17 @@ __device__ __forceinline__ float tri_test(float3 o, float3 w, float3 v0, float3 
 }
 
 // point scatterer: event at the closest approach t = (p - o).w when within r_s of the centre
+// The roundings are spelled out: whether a ray passes within r_s is a decision, and left to the
+// compiler's choice of fused products it changed with the code around it (6 of 16 million paths)
+__device__ __forceinline__ float dot3_rn(float3 a, float3 b) {
+  return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));
+}
 __device__ __forceinline__ float scat_test(float3 o, float3 w, float3 p, float rs2) {
   const float3 d = p - o;
-  const float t = dot3(d, w);
+  const float t = dot3_rn(d, w);
   if (!(t > T_MIN)) return -1.0f;
-  const float3 q = w * t - d;
-  return dot3(q, q) <= rs2 ? t : -1.0f;
+  const float3 q = f3(__fmaf_rn(w.x, t, -d.x), __fmaf_rn(w.y, t, -d.y), __fmaf_rn(w.z, t, -d.z));
+  return dot3_rn(q, q) <= rs2 ? t : -1.0f;
 }
 
 __device__ __forceinline__ bool hit_better(float t, uint32_t c, float tb, uint32_t cb) {

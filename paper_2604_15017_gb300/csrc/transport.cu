@@ -106,6 +106,15 @@ __global__ void __launch_bounds__(GEN_THREADS) k_generate_count(TransportArgs A,
     if (gen_h[b]) atomicAdd(&A.rk.cnt[b], gen_h[b]);
 }
 
+// Lanes of a warp that take work when n items are spread over `warps` resident warps: all 32 once
+// every warp has that many items, else as many as its share (at least WARP_LANES_MIN).  A pass
+// that does not fill the GPU lasts as long as its slowest warp, and a warp executes the union of
+// its lanes' branches: fewer lanes, shorter union.
+constexpr uint32_t WARP_LANES_MIN = 4;
+__device__ __forceinline__ uint32_t warp_lanes(uint32_t n, uint32_t warps) {
+  return min(32u, max(WARP_LANES_MIN, (n + warps - 1u) / warps));
+}
+
 // ------------------------------------------------------------------------------------------
 // Closest surface hit (transducer face, triangle BVH) of every live path, one ray per thread,
 // grid-stride.  The lanes of a warp start their rays at the root together, so the upper levels
@@ -116,8 +125,16 @@ __global__ void __launch_bounds__(TRAV_THREADS) k_traverse(TransportArgs A) {
   if (blockIdx.x == 0 && threadIdx.x == 0)  // secondary jobs of this round follow the previous rounds'
     A.cnt->nee_off[A.k] = A.k ? A.cnt->nee_off[A.k - 1] + A.cnt->nee[A.k - 1] : 0u;
   const uint32_t n = *A.trav_n;  // the rest of the queue carries its surface hit
+  // one wave of warps takes a small queue a few lanes each (warp_lanes); a larger one is walked
+  // grid-stride, consecutive rays in one block
+  const uint32_t warps = gridDim.x * (TRAV_THREADS / 32) / 2;  // the grid is two waves
+  const uint32_t lanes = warp_lanes(n, warps);
+  const uint32_t lane = threadIdx.x & 31u;
+  const bool spread = lanes < 32u;
+  uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (spread) i = lane < lanes ? (blockIdx.x + gridDim.x * (threadIdx.x >> 5)) * lanes + lane : n;
   bool overflow = false;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  for (; i < n; i += spread ? n : gridDim.x * blockDim.x) {
     const float4 pa = A.qin.pa[i];
     const float4 wt = A.qin.wt[i];
     const uint32_t prev = A.qin.meta[i].y;
@@ -134,100 +151,88 @@ __global__ void __launch_bounds__(TRAV_THREADS) k_traverse(TransportArgs A) {
 // uniform sphere grid, cells in the order the ray crosses them.  Every sphere whose
 // closest-approach point lies on the ray at parameter t is listed in the cell holding that
 // point, and that cell is entered at a parameter <= t, so a ray stops at the first cell it
-// would enter beyond its best hit.  Cell faces are computed from the grid origin at every step
-// (no accumulated increments).
+// would enter beyond its best hit.  The face ahead of step k along an axis lies at t_0 + k dt
+// (one FMA from the first face, no accumulated increments), and the ray leaves the grid at the
+// same expression's value for the last face, so a step that is taken stays inside the grid.
 //
 // Path lengths to the first event are spread roughly exponentially, so with one ray per thread
 // a warp would run as long as its longest ray with most lanes idle.  Instead every loop
-// iteration does the same work in every lane: enter one cell, test the two entries its 32-byte
-// record holds inline, step the DDA and read the next cell's record (entries past the second,
-// in crowded cells, take one iteration each).  Lanes whose rays have finished take the next
-// rays, once MARCH_REFILL_MIN of them wait, from a pool the warp claims in chunks of MARCH_CHUNK
-// consecutive (coherence-sorted) queue slots.
+// iteration does the same work in every lane: test the two entries of the lane's 32-byte
+// record, find the next record (a crowded cell's records are chained: the first names the
+// next) and start reading it.  Lanes whose rays have finished take the next rays, once
+// MARCH_REFILL_MIN of them wait, from a pool the warp claims in chunks of MARCH_CHUNK
+// consecutive (coherence-sorted) queue slots.  With few rays (a late round, a small pass) the
+// kernel lasts as long as its longest chain of iterations, so the rays are spread over all
+// resident warps, a few lanes each (warp_lanes).
+//
+// Bound by the latency of that chain: one L2 record read and ~70 instructions per iteration.  Per
+// inclusion frame (38M rays, 1.1e9 cells) closest hits took 19.3 ms when a crowded cell's entries
+// were looked up and tested one by one (its lanes' two further dependent reads held up the whole
+// warp in most iterations) and a step kept three cell coordinates; 16.6 ms so.  Five rounds of
+// 1e5 .. 1e4 rays: 1424 -> 790 us.
 // ------------------------------------------------------------------------------------------
 constexpr int MARCH_CHUNK = 64;
 constexpr int MARCH_REFILL_MIN = 8;
 
-__global__ void __launch_bounds__(MARCH_THREADS) k_march(TransportArgs A) {
+__global__ void __launch_bounds__(MARCH_THREADS, 8) k_march(TransportArgs A) {
   const SceneDev& S = A.S;
   const uint32_t n = A.cnt->live[A.k];
   if (S.n_scat == 0 || n == 0) return;
   uint32_t* claim = &A.cnt->march[A.k];
   const unsigned lane = threadIdx.x & 31u;
   const unsigned below = (1u << lane) - 1u;
-  const float h = S.gh, inv_h = 1.0f / h;
-  const float3 lo = S.glo;
+  const uint32_t warps = gridDim.x * (MARCH_THREADS / 32);
+  const uint32_t lanes = warp_lanes(n, warps);
+  const uint32_t lane_mask = lanes >= 32u ? 0xFFFFFFFFu : (1u << lanes) - 1u;
+  const uint32_t chunk = lanes >= 32u ? (uint32_t)MARCH_CHUNK : lanes;
+  const int refill_min = min(MARCH_REFILL_MIN, (int)lanes);
+  const float h = S.gh;
   const int nx = S.gnx, ny = S.gny, nz = S.gnz;
-  const int dy = nx, dz = nx * ny;
   // lane state
   uint32_t ray = 0xFFFFFFFFu;  // queue slot of the current ray; none when 0xFFFFFFFF
   float3 o = f3(0.0f, 0.0f, 0.0f), w = o;
-  float ix = 0.0f, iy = 0.0f, iz = 0.0f, tnx = 0.0f, tny = 0.0f, tnz = 0.0f, tbest = 0.0f, t0hit = 0.0f;
-  uint32_t prev = 0u, cbest = 0u, code0 = 0u, e = 0u, e_end = 0u;
-  int cx = 0, cy = 0, cz = 0, idx = 0, sx = 1, sy = 1, sz = 1, ux = 0, uy = 0, uz = 0;
-  // The DDA runs one cell ahead: (cx, cy, cz, idx) is the next cell to enter, at t_ahead, and
-  // its inline record (first two entries) is read as soon as the DDA gets there, so the read has
-  // an iteration to arrive.  It is read only while t_ahead <= tbest; tbest only decreases, so a
-  // record not read is a record never needed.
-  float t_ahead = 0.0f;
-  bool ahead_ok = false;
-  float4 slot_a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), slot_b = slot_a;
-  auto fetch_ahead = [&]() {
-    if (ahead_ok && t_ahead <= tbest) {
-      slot_a = __ldg(&S.cell2[2 * idx]);
-      slot_b = __ldg(&S.cell2[2 * idx + 1]);
-    } else {
-      slot_a.w = slot_b.w = 0.0f;
-    }
-  };
-  auto step_ahead = [&]() {
-    if (tnx <= tny && tnx <= tnz) {
-      t_ahead = tnx;
-      cx += sx;
-      idx += sx;
-      ahead_ok = (unsigned)cx < (unsigned)nx;
-      tnx = (fmaf((float)(cx + ux), h, lo.x) - o.x) * ix;
-    } else if (tny <= tnz) {
-      t_ahead = tny;
-      cy += sy;
-      idx += sy * dy;
-      ahead_ok = (unsigned)cy < (unsigned)ny;
-      tny = (fmaf((float)(cy + uy), h, lo.y) - o.y) * iy;
-    } else {
-      t_ahead = tnz;
-      cz += sz;
-      idx += sz * dz;
-      ahead_ok = (unsigned)cz < (unsigned)nz;
-      tnz = (fmaf((float)(cz + uz), h, lo.z) - o.z) * iz;
-    }
-    fetch_ahead();
+  // per axis: the next face (tn = fma(k, dt, t_0)), its step number k, dt, t_0, the cell stride
+  float tnx = 0.0f, tny = 0.0f, tnz = 0.0f, kx = 0.0f, ky = 0.0f, kz = 0.0f;
+  float dtx = 0.0f, dty = 0.0f, dtz = 0.0f, fx = 0.0f, fy = 0.0f, fz = 0.0f;
+  int sx = 0, sy = 0, sz = 0, cell = 0;
+  float tbest = 0.0f, tend = 0.0f, t0hit = 0.0f;
+  uint32_t prev = 0u, cbest = 0u, code0 = 0u;
+  float4 slot_a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), slot_b = slot_a;  // the record to test next
+  auto fetch = [&](int rec) {
+    slot_a = __ldg(&S.cell_rec[2 * (size_t)rec]);
+    slot_b = __ldg(&S.cell_rec[2 * (size_t)rec + 1]);
   };
   auto test = [&](float4 sp) {
-    const uint32_t code = __float_as_uint(sp.w) & 0x7FFFFFFFu;
-    const float t = code == 0u || code == prev ? -1.0f : scat_test(o, w, xyz(sp), S.rs2);
-    if (t > 0.0f && hit_better(t, code, tbest, cbest)) {
+    const uint32_t id = __float_as_uint(sp.w) & 0xFFFFFu;
+    const float t = scat_test(o, w, xyz(sp), S.rs2);
+    const uint32_t code = prim_code(CLS_SCAT, id);
+    if (t > 0.0f && code != prev && hit_better(t, code, tbest, cbest)) {
       tbest = t;
       cbest = code;
     }
   };
-  uint32_t pool = 0u, pool_end = 0u;  // warp-uniform
-  bool exhausted = false;             // warp-uniform
+  // the first chunk of every warp is its own; the counter hands out the ones after those
+  uint32_t pool = min(n, (blockIdx.x + gridDim.x * (threadIdx.x >> 5)) * chunk);  // warp-uniform
+  uint32_t pool_end = min(n, pool + chunk);
+  bool exhausted = pool >= n;  // warp-uniform
   while (true) {
-    // hand the pool's rays to idle lanes once MARCH_REFILL_MIN of them wait, so that the setup
-    // of new rays runs on many lanes at once; rays that miss the grid leave their lane idle
-    uint32_t idle = __ballot_sync(0xFFFFFFFFu, ray == 0xFFFFFFFFu);
-    if (__popc(idle) < MARCH_REFILL_MIN) idle = 0u;
+    // hand the pool's rays to idle lanes once refill_min of them wait, so that the setup of new
+    // rays runs on many lanes at once; rays that miss the grid leave their lane idle
+    uint32_t idle = __ballot_sync(0xFFFFFFFFu, ray == 0xFFFFFFFFu) & lane_mask;
+    if (__popc(idle) < refill_min) idle = 0u;
     while (idle && !exhausted) {
       if (pool == pool_end) {
-        uint32_t b = 0u;
-        if (lane == 0) b = atomicAdd(claim, (uint32_t)MARCH_CHUNK);
-        b = __shfl_sync(0xFFFFFFFFu, b, 0);
+        uint32_t b = warps * chunk;
+        if (b < n) {
+          if (lane == 0) b += atomicAdd(claim, chunk);
+          b = __shfl_sync(0xFFFFFFFFu, b, 0);
+        }
         if (b >= n) {
           exhausted = true;
           break;
         }
         pool = b;
-        pool_end = min(b + (uint32_t)MARCH_CHUNK, n);
+        pool_end = min(b + chunk, n);
       }
       const uint32_t take = min((uint32_t)__popc(idle), pool_end - pool);
       const uint32_t rank = __popc(idle & below);
@@ -241,9 +246,9 @@ __global__ void __launch_bounds__(MARCH_THREADS) k_march(TransportArgs A) {
         prev = A.qin.meta[ray].y;
         tbest = t0hit = hit.x;
         cbest = code0 = __float_as_uint(hit.y);
-        ix = safe_inv(w.x);
-        iy = safe_inv(w.y);
-        iz = safe_inv(w.z);
+        const float ix = safe_inv(w.x), iy = safe_inv(w.y), iz = safe_inv(w.z);
+        const float3 lo = S.glo;
+        // the grid's slabs: t of the low faces and of the far ones
         const float ax = (lo.x - o.x) * ix, bx = (fmaf((float)nx, h, lo.x) - o.x) * ix;
         const float ay = (lo.y - o.y) * iy, by = (fmaf((float)ny, h, lo.y) - o.y) * iy;
         const float az = (lo.z - o.z) * iz, bz = (fmaf((float)nz, h, lo.z) - o.z) * iz;
@@ -252,54 +257,72 @@ __global__ void __launch_bounds__(MARCH_THREADS) k_march(TransportArgs A) {
         if (t0 > t1) {
           ray = 0xFFFFFFFFu;  // misses the grid before its surface hit: nothing to do
         } else {
-          cx = min(nx - 1, max(0, (int)floorf((fmaf(w.x, t0, o.x) - lo.x) * inv_h)));
-          cy = min(ny - 1, max(0, (int)floorf((fmaf(w.y, t0, o.y) - lo.y) * inv_h)));
-          cz = min(nz - 1, max(0, (int)floorf((fmaf(w.z, t0, o.z) - lo.z) * inv_h)));
-          sx = w.x > 0.0f ? 1 : -1;
-          sy = w.y > 0.0f ? 1 : -1;
-          sz = w.z > 0.0f ? 1 : -1;
-          ux = w.x > 0.0f;
-          uy = w.y > 0.0f;
-          uz = w.z > 0.0f;
-          tnx = w.x == 0.0f ? 3.0e38f : (fmaf((float)(cx + ux), h, lo.x) - o.x) * ix;
-          tny = w.y == 0.0f ? 3.0e38f : (fmaf((float)(cy + uy), h, lo.y) - o.y) * iy;
-          tnz = w.z == 0.0f ? 3.0e38f : (fmaf((float)(cz + uz), h, lo.z) - o.z) * iz;
-          idx = (cz * ny + cy) * nx + cx;
-          t_ahead = t0;  // the first cell is the one ahead
-          ahead_ok = true;
-          e = e_end = 0u;
-          fetch_ahead();
+          const float inv_h = 1.0f / h;
+          const int cx = min(nx - 1, max(0, (int)floorf((fmaf(w.x, t0, o.x) - lo.x) * inv_h)));
+          const int cy = min(ny - 1, max(0, (int)floorf((fmaf(w.y, t0, o.y) - lo.y) * inv_h)));
+          const int cz = min(nz - 1, max(0, (int)floorf((fmaf(w.z, t0, o.z) - lo.z) * inv_h)));
+          // upward along an axis when its inverse is positive (so also for a direction of +0,
+          // whose faces then lie at huge t)
+          const bool ux = ix > 0.0f, uy = iy > 0.0f, uz = iz > 0.0f;
+          // clamped so that k dt + t_0 stays ordered in k, whatever the coordinates' scale
+          dtx = fminf(h * fabsf(ix), 1e30f);
+          dty = fminf(h * fabsf(iy), 1e30f);
+          dtz = fminf(h * fabsf(iz), 1e30f);
+          tnx = fx = fmaxf((fmaf((float)(cx + (ux ? 1 : 0)), h, lo.x) - o.x) * ix, -3e38f);
+          tny = fy = fmaxf((fmaf((float)(cy + (uy ? 1 : 0)), h, lo.y) - o.y) * iy, -3e38f);
+          tnz = fz = fmaxf((fmaf((float)(cz + (uz ? 1 : 0)), h, lo.z) - o.z) * iz, -3e38f);
+          // past the last face along an axis the ray is outside: no cell is entered at or after
+          // tend, and t_0 + k dt < tend only for faces before the last
+          tend = fminf(fminf(fmaf((float)(ux ? nx - 1 - cx : cx), dtx, fx), fmaf((float)(uy ? ny - 1 - cy : cy), dty, fy)),
+                       fmaf((float)(uz ? nz - 1 - cz : cz), dtz, fz));
+          kx = ky = kz = 0.0f;
+          sx = ux ? 1 : -1;
+          sy = uy ? nx : -nx;
+          sz = uz ? nx * ny : -nx * ny;
+          cell = (cz * ny + cy) * nx + cx;
+          fetch(cell);
         }
       }
       pool += take;
-      idle = __ballot_sync(0xFFFFFFFFu, ray == 0xFFFFFFFFu);
+      idle = __ballot_sync(0xFFFFFFFFu, ray == 0xFFFFFFFFu) & lane_mask;
     }
     if (__all_sync(0xFFFFFFFFu, ray == 0xFFFFFFFFu)) break;  // pool exhausted, every lane idle
     if (ray == 0xFFFFFFFFu) continue;
-    if (e < e_end) {  // entries past the first two of a crowded cell
-      test(__ldg(&S.cell_sph[e]));
-      ++e;
-      continue;
-    }
-    if (!(ahead_ok && t_ahead <= tbest)) {  // no cell left to enter below tbest: done
-      if (cbest != code0) {  // a scatterer comes first; its pass-through carries the surface hit on
-        A.keep[ray] = make_float2(t0hit, __uint_as_float(code0));  // the hit this ray came with
-        A.hits[ray] = make_float2(tbest, __uint_as_float(cbest));
+    test(slot_a);
+    test(slot_b);
+    // the record after this one: the next of a crowded cell's chain, or the next cell's
+    int rec = (int)((__float_as_uint(slot_a.w) >> 20 << 12) | (__float_as_uint(slot_b.w) >> 20));
+    if (rec != 0) {
+      rec += nx * ny * nz - 1;
+    } else {
+      float t;
+      if (tnx <= tny && tnx <= tnz) {
+        t = tnx;
+        cell += sx;
+        kx += 1.0f;
+        tnx = fmaf(kx, dtx, fx);
+      } else if (tny <= tnz) {
+        t = tny;
+        cell += sy;
+        ky += 1.0f;
+        tny = fmaf(ky, dty, fy);
+      } else {
+        t = tnz;
+        cell += sz;
+        kz += 1.0f;
+        tnz = fmaf(kz, dtz, fz);
       }
-      ray = 0xFFFFFFFFu;
-      continue;
+      if (!(t <= tbest && t < tend)) {  // no cell left to enter below tbest: done
+        if (cbest != code0) {  // a scatterer comes first; its pass-through carries the surface hit on
+          A.keep[ray] = make_float2(t0hit, __uint_as_float(code0));  // the hit this ray came with
+          A.hits[ray] = make_float2(tbest, __uint_as_float(cbest));
+        }
+        ray = 0xFFFFFFFFu;
+        continue;
+      }
+      rec = cell;
     }
-    // enter the cell ahead: test its inline entries, then step the DDA past it
-    const float4 a = slot_a, b = slot_b;
-    const int cell = idx;
-    test(a);
-    test(b);
-    if (__float_as_uint(b.w) >> 31) {
-      const uint32_t word = __ldg(&S.cell[cell]);
-      e = (word >> 8) + 2u;
-      e_end = (word >> 8) + (word & 0xFFu);
-    }
-    step_ahead();
+    fetch(rec);
   }
 }
 

@@ -89,9 +89,8 @@ struct SceneDev {
                              // n2=(c0 z, c1 z) n3=int4(child0, child1, count0, count1)
   const float4* prims_t;     // triangles in leaf order: (v0, code) (e1, -) (e2, -)
   const float4* nodes4;      // the triangle tree as a 4-wide BVH (8 float4 per node, same leaves)
-  const uint32_t* cell;        // scatterer grid, per cell (z * gny + y) * gnx + x: first entry << 8 | count
-  const float4* cell_sph;      // per (cell, sphere): (centre, bits(code))
-  const float4* cell2;         // per cell its first two entries; code 0: empty, bit 31: more follow
+  const float4* cell_rec;      // scatterer grid: records of two entries (centre, id | next bits << 20),
+                               // cell (z * gny + y) * gnx + x first, then the crowded cells' chains
   float3 glo;                  // grid origin and cell edge
   float gh;
   int gnx, gny, gnz;
