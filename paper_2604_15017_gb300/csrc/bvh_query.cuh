@@ -91,18 +91,26 @@ __device__ __forceinline__ void xdcr_test(const Acq& q, float3 o, float3 w, floa
   }
 }
 
+// Two triangles at a time, all their loads first: a triangle used to cost two dependent reads (its
+// id, then the rest), one triangle after the other, for every lane of a warp that sat in a leaf
+// (closest hits per inclusion frame 16.6 -> 16.3 ms, five rounds of 1e5 .. 1e4 rays 790 -> 716 us,
+// with the two leaves of a node in one loop).
 __device__ __forceinline__ void leaf_closest(const SceneDev& S, int first, int count, float3 o, float3 w,
                                              uint32_t prev, float& tbest, uint32_t& cbest) {
-  for (int i = first; i < first + count; ++i) {
-    const float4 A = __ldg(&S.prims_t[3 * i]);
-    const uint32_t code = __float_as_uint(A.w);
-    if (code == prev) continue;
-    const float4 B = __ldg(&S.prims_t[3 * i + 1]);
-    const float4 C = __ldg(&S.prims_t[3 * i + 2]);
-    const float t = tri_test(o, w, xyz(A), xyz(B), xyz(C));
-    if (t > 0.0f && hit_better(t, code, tbest, cbest)) {
-      tbest = t;
-      cbest = code;
+  for (int i = first; i < first + count; i += 2) {
+    const int j = min(i + 1, first + count - 1);  // an odd leaf tests its last triangle twice
+    const float4 A0 = __ldg(&S.prims_t[3 * i]), B0 = __ldg(&S.prims_t[3 * i + 1]), C0 = __ldg(&S.prims_t[3 * i + 2]);
+    const float4 A1 = __ldg(&S.prims_t[3 * j]), B1 = __ldg(&S.prims_t[3 * j + 1]), C1 = __ldg(&S.prims_t[3 * j + 2]);
+    const uint32_t c0 = __float_as_uint(A0.w), c1 = __float_as_uint(A1.w);
+    const float t0 = tri_test(o, w, xyz(A0), xyz(B0), xyz(C0));
+    const float t1 = tri_test(o, w, xyz(A1), xyz(B1), xyz(C1));
+    if (t0 > 0.0f && c0 != prev && hit_better(t0, c0, tbest, cbest)) {
+      tbest = t0;
+      cbest = c0;
+    }
+    if (t1 > 0.0f && c1 != prev && hit_better(t1, c1, tbest, cbest)) {
+      tbest = t1;
+      cbest = c1;
     }
   }
 }
@@ -128,16 +136,12 @@ __device__ __forceinline__ void tri_closest(const SceneDev& S, float3 o, float3 
       bool h0, h1;
       float t0, t1;
       node_boxes(r, n0, n1, n2, tbest, h0, h1, t0, t1);
-      if (h0 && n3.z > 0) {
-        leaf_closest(S, n3.x, n3.z, o, w, prev, tbest, cbest);
-        h0 = false;
-      }
-      if (h1 && n3.w > 0) {
-        leaf_closest(S, n3.y, n3.w, o, w, prev, tbest, cbest);
-        h1 = false;
-      }
-      h0 = h0 && n3.x >= 0;
-      h1 = h1 && n3.y >= 0;
+      // the triangles of two leaf children are adjacent in leaf order: one loop serves the lanes
+      // whose left, right or both children are leaves
+      const bool l0 = h0 && n3.z > 0, l1 = h1 && n3.w > 0;
+      if (l0 || l1) leaf_closest(S, l0 ? n3.x : n3.y, (l0 ? n3.z : 0) + (l1 ? n3.w : 0), o, w, prev, tbest, cbest);
+      h0 = h0 && n3.z == 0 && n3.x >= 0;
+      h1 = h1 && n3.w == 0 && n3.y >= 0;
       if (h0 && h1) {
         const bool first0 = t0 <= t1;
         if (sp < BVH_STACK) {
