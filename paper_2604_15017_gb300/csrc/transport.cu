@@ -109,8 +109,9 @@ __global__ void __launch_bounds__(GEN_THREADS) k_generate_count(TransportArgs A,
 // Lanes of a warp that take work when n items are spread over `warps` resident warps: all 32 once
 // every warp has that many items, else as many as its share (at least WARP_LANES_MIN).  A pass
 // that does not fill the GPU lasts as long as its slowest warp, and a warp executes the union of
-// its lanes' branches: fewer lanes, shorter union.
-constexpr uint32_t WARP_LANES_MIN = 4;
+// its lanes' branches: fewer lanes, shorter union.  At least 8 (with 4, late rounds that run
+// beside the secondary rays found no room for their many warps: frame +0.45 ms).
+constexpr uint32_t WARP_LANES_MIN = 8;
 __device__ __forceinline__ uint32_t warp_lanes(uint32_t n, uint32_t warps) {
   return min(32u, max(WARP_LANES_MIN, (n + warps - 1u) / warps));
 }
@@ -121,7 +122,7 @@ __device__ __forceinline__ uint32_t warp_lanes(uint32_t n, uint32_t warps) {
 // of the BVH are fetched once per warp.  The scatterers are searched next by k_march below the
 // distance written here.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(TRAV_THREADS) k_traverse(TransportArgs A) {
+__global__ void __launch_bounds__(TRAV_THREADS, 8) k_traverse(TransportArgs A) {
   if (blockIdx.x == 0 && threadIdx.x == 0)  // secondary jobs of this round follow the previous rounds'
     A.cnt->nee_off[A.k] = A.k ? A.cnt->nee_off[A.k - 1] + A.cnt->nee[A.k - 1] : 0u;
   const uint32_t n = *A.trav_n;  // the rest of the queue carries its surface hit
@@ -171,8 +172,10 @@ __global__ void __launch_bounds__(TRAV_THREADS) k_traverse(TransportArgs A) {
 // warp in most iterations) and a step kept three cell coordinates; 16.6 ms so.  Five rounds of
 // 1e5 .. 1e4 rays: 1424 -> 790 us.
 // ------------------------------------------------------------------------------------------
-constexpr int MARCH_CHUNK = 64;
-constexpr int MARCH_REFILL_MIN = 8;
+// 32-ray claims and a refill at 4 idle lanes, measured against 64 and 128 rays, 8, 12 and 16 lanes
+// (medium render 927 us of closest hits against 977 with 64-ray claims; the frame is indifferent)
+constexpr int MARCH_CHUNK = 32;
+constexpr int MARCH_REFILL_MIN = 4;
 
 __global__ void __launch_bounds__(MARCH_THREADS, 8) k_march(TransportArgs A) {
   const SceneDev& S = A.S;
