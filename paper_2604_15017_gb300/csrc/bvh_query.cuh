@@ -250,34 +250,40 @@ __device__ __forceinline__ bool xtrav_step(const SceneDev& S, float3 o, float3 d
   bool h[4];
   node4_boxes(T.r, n, T.tmax, tn, h);
   const int ch[4] = {n.ch.x, n.ch.y, n.ch.z, n.ch.w}, cn[4] = {n.cn.x, n.cn.y, n.cn.z, n.cn.w};
-  int next = -1;
+  int next = -1, m[4];
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    if (!h[c]) continue;
-    if (cn[c] > 0) {
-      for (int i = ch[c]; i < ch[c] + cn[c]; ++i) {
-        const float4 A = __ldg(&S.prims_t[3 * i]);
-        const uint32_t code = __float_as_uint(A.w);
-        const float4 B = __ldg(&S.prims_t[3 * i + 1]);
-        const float4 C = __ldg(&S.prims_t[3 * i + 2]);
-        const float t = tri_test(o, d, xyz(A), xyz(B), xyz(C));
-        if (t > 0.0f && t < T.tmax && code_id(code) != T.skip) {
-          if (T.n < MAX_XINGS) {
-            xt[T.n] = t;
-            xid[T.n] = code_id(code);
-            ++T.n;
-          } else {
-            T.overflow = true;
-          }
-        }
-      }
-    } else if (ch[c] >= 0) {
-      if (next < 0) {
-        next = ch[c];
-      } else if (T.sp < BVH_STACK) {
-        stack[T.sp++] = ch[c];
+    m[c] = h[c] ? cn[c] : 0;  // triangles of a hit leaf child
+    if (!h[c] || cn[c] > 0 || ch[c] < 0) continue;
+    if (next < 0) {
+      next = ch[c];
+    } else if (T.sp < BVH_STACK) {
+      stack[T.sp++] = ch[c];
+    }
+  }
+  // the triangles of all hit leaves in one loop (lanes whose leaves sit in different slots test
+  // theirs together), two at a time with all their loads first
+  const int e1 = m[0] + m[1], e2 = e1 + m[2], total = e2 + m[3];
+  auto tri_at = [&](int k) { return k < e1 ? (k < m[0] ? ch[0] + k : ch[1] + (k - m[0])) : (k < e2 ? ch[2] + (k - e1) : ch[3] + (k - e2)); };
+  auto keep = [&](float t, uint32_t code) {
+    if (t > 0.0f && t < T.tmax && code_id(code) != T.skip) {
+      if (T.n < MAX_XINGS) {
+        xt[T.n] = t;
+        xid[T.n] = code_id(code);
+        ++T.n;
+      } else {
+        T.overflow = true;
       }
     }
+  };
+  for (int k = 0; k < total; k += 2) {
+    const bool two = k + 1 < total;
+    const int i = tri_at(k), j = two ? tri_at(k + 1) : i;
+    const float4 A0 = __ldg(&S.prims_t[3 * i]), B0 = __ldg(&S.prims_t[3 * i + 1]), C0 = __ldg(&S.prims_t[3 * i + 2]);
+    const float4 A1 = __ldg(&S.prims_t[3 * j]), B1 = __ldg(&S.prims_t[3 * j + 1]), C1 = __ldg(&S.prims_t[3 * j + 2]);
+    keep(tri_test(o, d, xyz(A0), xyz(B0), xyz(C0)), __float_as_uint(A0.w));
+    const float t1 = tri_test(o, d, xyz(A1), xyz(B1), xyz(C1));
+    if (two) keep(t1, __float_as_uint(A1.w));
   }
   if (next >= 0) {
     T.node = next;
