@@ -52,7 +52,6 @@ void launch_active_paths(const uint32_t* record, uint32_t n_paths, int kmax, uin
                          const float4* tri_nrm = nullptr);
 void launch_path_adjoint(const AdjArgs& a, int grid, cudaStream_t st);
 cudaError_t adjoint_set_attrs();
-void launch_grad_reduce(const float* gpart, int nblocks, int P, float* g, cudaStream_t st);
 // columns [0, Ps) of gpart to g, the others to g2 (added to it when acc2)
 void launch_grad_reduce_split(const float* gpart, int nblocks, int P, int Ps, float* g, float* g2, int acc2,
                               cudaStream_t st);
