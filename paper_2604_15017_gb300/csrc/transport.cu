@@ -702,6 +702,7 @@ __global__ void __launch_bounds__(NEE_THREADS) k_nee(TransportArgs A) {
 // ------------------------------------------------------------------------------------------
 
 constexpr int RS_THREADS = 512;
+static_assert(RAY_BUCKETS <= COUNT_SCAN_MAX, "the ray sort's counts fit one scan");
 constexpr int JOB_BUCKETS = 4096;  // <= RAY_BUCKETS (the job sort's scratch is sized as the ray sort's)
 // items per thread and chunk, measured: 1024-ray chunks for the rays (512: +0.25 ms of sort per
 // frame, 2048: +0.12 ms, 8192: +0.5 ms), 2048-job chunks for the jobs
