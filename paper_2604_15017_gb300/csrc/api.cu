@@ -611,7 +611,7 @@ int do_bmode(us_ctx* ctx, const Acq& q, const Img& im, const float* rf, float* b
   CKS(ws(ctx, W_KEY, 2, st, &key));
   {
     StageScope sc_(ctx, US_STAGE_DAS, 1, st);
-    launch_das(q, im, rf, irf, grid_of(ctx, 8), st, ctx->opts[US_OPT_DAS_TMA] ? ctx->d_status : nullptr);
+    launch_das(q, im, rf, irf, st, ctx->opts[US_OPT_DAS_TMA] ? ctx->d_status : nullptr);
   }
   irf_made(ctx, q, im, rf, irf);
   {
@@ -1023,7 +1023,7 @@ int us_das(us_ctx* ctx, const us_acq_desc* acq, const us_img_desc* img, const fl
   CKS(make_img(ctx, img, im));
   if (!rf_dev || !irf_dev) return fail(ctx, US_ERR_ARG, "null buffer");
   StageScope sc_(ctx, US_STAGE_DAS, 1, (cudaStream_t)stream);
-  launch_das(q, im, rf_dev, irf_dev, grid_of(ctx, 8), (cudaStream_t)stream,
+  launch_das(q, im, rf_dev, irf_dev, (cudaStream_t)stream,
              ctx->opts[US_OPT_DAS_TMA] ? ctx->d_status : nullptr);
   CK(cudaGetLastError());
   return US_OK;
@@ -1128,7 +1128,7 @@ static int bmode_vjp(us_ctx* ctx, const us_acq_desc* acq, const us_img_desc* img
   const IrfKey& k = ctx->L->ikey;
   if (!(reuse_irf && k.valid && k.rf == rf_dev && k.irf == irf && k.sig == das_signature(q, im))) {
     StageScope sc_(ctx, US_STAGE_DAS, 1, st);
-    launch_das(q, im, rf_dev, irf, grid_of(ctx, 8), st, ctx->opts[US_OPT_DAS_TMA] ? ctx->d_status : nullptr);
+    launch_das(q, im, rf_dev, irf, st, ctx->opts[US_OPT_DAS_TMA] ? ctx->d_status : nullptr);
     irf_made(ctx, q, im, rf_dev, irf);
   }
   unsigned long long* acc;

@@ -41,11 +41,31 @@ __device__ __forceinline__ ff das_utx(const Acq& q, const DasGeo& g, ff x, ff z,
   p = ff_addx(p, ff_mulf(g.half_w, fabsf(st)));
   return ff_mul(p, g.k);
 }
-__device__ __forceinline__ ff das_urx(const Acq& q, const DasGeo& g, ff x, ff z, int e) {
-  const ff xe = ff_mulf(ff{(float)e - 0.5f * (float)(q.ne - 1), 0.0f}, q.pitch);
-  const ff dx = ff_addx(x, ff{-xe.hi, -xe.lo});
-  const ff r2 = ff_addx(ff_mul(dx, dx), ff_mul(z, z));
-  return ff_mul(ff_sqrt(r2), g.k);
+// Receive side, in samples: the pixel's lateral position and squared depth and the element's
+// position are scaled by fs / c_bf once, so that a (pixel, element) pair costs one difference, one
+// square, one sum and a square root refined by its exact residual (relative error 2^-45): ~40
+// instructions where the unscaled form, with an IEEE root and divide, took ~110.
+struct DasRx {
+  ff x;   // x fs / c_bf
+  ff z2;  // (z fs / c_bf)^2
+};
+__device__ __forceinline__ DasRx das_rx(const DasGeo& g, ff x, ff z) {
+  const ff zk = ff_mul(z, g.k);
+  return DasRx{ff_mul(x, g.k), ff_mul(zk, zk)};
+}
+__device__ __forceinline__ ff das_elem(const Acq& q, const DasGeo& g, int e) {  // x_e fs / c_bf
+  return ff_mul(ff_mulf(ff{(float)e - 0.5f * (float)(q.ne - 1), 0.0f}, q.pitch), g.k);
+}
+__device__ __forceinline__ ff das_urx(const DasRx& p, ff xe) {
+  const ff dx = ff_addx(p.x, ff{-xe.hi, -xe.lo});
+  const float h = __fmul_rn(dx.hi, dx.hi);
+  const float l = __fmaf_rn(__fmul_rn(2.0f, dx.hi), dx.lo, __fmaf_rn(dx.hi, dx.hi, -h));
+  const ff s = ff_two_sum(h, p.z2.hi);
+  const float r2 = fmaxf(s.hi, 1e-30f);  // a pixel on the element: 1e-15 samples
+  const float inv = rsqrtf(r2);
+  const float r = __fmul_rn(r2, inv);
+  const float res = __fadd_rn(__fmaf_rn(-r, r, r2), __fadd_rn(s.lo, __fadd_rn(l, p.z2.lo)));
+  return ff{r, __fmul_rn(res, __fmul_rn(0.5f, inv))};
 }
 __device__ __forceinline__ float hann_w(int e, int ne) {
   return 0.5f * (1.0f - cospif(2.0f * (float)(e + 1) / (float)(ne + 1)));
@@ -86,48 +106,104 @@ __device__ __forceinline__ void das_tap(float2 a, float2 b, int& i, float& f) {
   }
 }
 
-// DAS: one pixel per thread; transmit delays staged per pixel in shared memory, the receive
-// delay computed once per (pixel, element) and reused for every transmit; channel data read
-// through the read-only path (rows stay L2-resident)
+// DAS.  A block owns a tile of DAS_TL lines x DAS_TD depths; a warp covers 8 lines x 4 depths.
+// Bound by the L1's gathers: neighbouring depths are ~3 samples apart, neighbouring lines less than
+// one on average, so a warp of 32 depths read 4 lines of 128 bytes per load and 12 bytes per tap
+// from the L2, an 8 x 4 patch reads 1-2 lines and ~2.5 bytes per tap.  The transmit delays are
+// staged per pixel in shared memory, their row offsets folded in; the receive delay serves all
+// transmits of an element; taps are checked against the record once per (pixel, element), by
+// the pixel's smallest and largest transmit delay.  The elements of a chunk are shared out over
+// DAS_ES groups of threads, so that small images fill the GPU too; a pixel's sums over the
+// transmits meet in shared memory and are weighted and added in element order by one thread.
+// 128 elements, 256 x 1024 pixels: 16 transmits 921 -> 378 us (5.4e8 taps), 1 transmit 239 ->
+// 133 us (there the delays, 3.4e7 of them, are most of it).  Elements split two ways instead of four,
+// patches of 16 x 2 and 4 x 8: equal or slower.
 constexpr int DAS_THREADS = 256;
+constexpr int DAS_ES = 4, DAS_TL = 8, DAS_TD = 8, DAS_PX = DAS_TL * DAS_TD;
+constexpr int DAS_EC = 32;  // elements per chunk
+static_assert(DAS_PX * DAS_ES == DAS_THREADS && DAS_TL == 8 && DAS_EC % DAS_ES == 0, "a warp is 8 lines x 4 depths");
+__host__ __device__ constexpr size_t das_smem(int ne, int ntx, bool dynamic) {
+  return sizeof(float2) * ((size_t)ntx * DAS_PX + ne) + sizeof(float) * (ne + (dynamic ? 4 : 2) * DAS_EC * DAS_PX);
+}
 __global__ void __launch_bounds__(DAS_THREADS) k_das(Acq q, Img im, const float* __restrict__ rf,
                                                      float* __restrict__ irf) {
-  extern __shared__ float2 utx_s[];  // [ntx][DAS_THREADS]
-  const int npx = im.nl * im.nd;
+  extern __shared__ float2 das_sm[];
+  float2* utx_s = das_sm;                                     // [ntx][DAS_PX]: (first sample + row offset, fraction)
+  float2* xe_s = das_sm + q.ntx * DAS_PX;                     // [ne] element positions (float-float)
+  float* w_s = reinterpret_cast<float*>(xe_s + q.ne);         // [ne] Hann weights
+  float* s_s = w_s + q.ne;                                    // [2][DAS_EC][DAS_PX] sums over the transmits
+  float* wd_s = s_s + 2 * DAS_EC * DAS_PX;                    // the same of the dynamic aperture's weights
   const DasGeo g = das_geo(q);
-  for (int base = blockIdx.x * DAS_THREADS; base < npx; base += gridDim.x * DAS_THREADS) {
-    const int p = base + threadIdx.x;
-    const bool valid = p < npx;
-    const int l = valid ? p / im.nd : 0, d = valid ? p - l * im.nd : 0;
-    const ff x = grid_coord(im.x0, im.x1, l, im.nl), z = grid_coord(im.z0, im.z1, d, im.nd);
-    for (int t = 0; t < q.ntx; ++t) utx_s[t * DAS_THREADS + threadIdx.x] = das_split(das_utx(q, g, x, z, t));
-    float acc = 0.0f;
-    if (valid) {
-      const size_t tstride = (size_t)q.ne * q.ns;  // between one element's rows of two transmits
-      for (int e = 0; e < q.ne; ++e) {
-        const float2 ur = das_split(das_urx(q, g, x, z, e));
-        const float* row = rf + (size_t)e * q.ns;
-        float s = 0.0f;
+  const int tiles_d = (im.nd + DAS_TD - 1) / DAS_TD;
+  const int tl = blockIdx.x / tiles_d;
+  const int px = threadIdx.x % DAS_PX, es = threadIdx.x / DAS_PX;
+  const int l = tl * DAS_TL + (px & 7), d = (blockIdx.x - tl * tiles_d) * DAS_TD + (px >> 3);
+  const bool valid = l < im.nl && d < im.nd;
+  const ff x = grid_coord(im.x0, im.x1, min(l, im.nl - 1), im.nl), z = grid_coord(im.z0, im.z1, min(d, im.nd - 1), im.nd);
+  const int tstride = q.ne * q.ns;  // between one element's rows of two transmits
+  for (int t = es; t < q.ntx; t += DAS_ES) {
+    const float2 u = das_split(das_utx(q, g, x, z, t));
+    utx_s[t * DAS_PX + px] = make_float2(__int_as_float(__float_as_int(u.x) + t * tstride), u.y);
+  }
+  for (int e = threadIdx.x; e < q.ne; e += DAS_THREADS) {
+    const ff xe = das_elem(q, g, e);
+    xe_s[e] = make_float2(xe.hi, xe.lo);
+    w_s[e] = hann_w(e, q.ne);
+  }
+  __syncthreads();
+  int imin = 0x7FFFFFFF, imax = -0x7FFFFFFF;
+  for (int t = 0; t < q.ntx; ++t) {
+    const int i = __float_as_int(utx_s[t * DAS_PX + px].x) - t * tstride;
+    imin = min(imin, i);
+    imax = max(imax, i);
+  }
+  // clamped so that no sum below overflows, and none of clamped values passes the check
+  imin = max(-(1 << 22), min(imin, 1 << 22));
+  imax = max(-(1 << 22), min(imax, 1 << 22));
+  const DasRx p = das_rx(g, x, z);
+  const bool dynamic = im.fnum > 0.0f;
+  float acc = 0.0f;
+  for (int e0 = 0, buf = 0; e0 < q.ne; e0 += DAS_EC, buf ^= 1) {
+    const int e1 = min(e0 + DAS_EC, q.ne);
+    float* sb = s_s + buf * DAS_EC * DAS_PX + px;
+    float* wb = wd_s + buf * DAS_EC * DAS_PX + px;
+    for (int e = e0 + es; e < e1; e += DAS_ES) {
+      const float2 xe = xe_s[e];
+      const float2 ur = das_split(das_urx(p, ff{xe.x, xe.y}));
+      const int ir = __float_as_int(ur.x);
+      const float2 b = make_float2(__int_as_float(ir + e * q.ns), ur.y);
+      float s = 0.0f;
+      const int irc = max(-(1 << 24), min(ir, 1 << 24));
+      if (irc + imin >= 0 && irc + imax + 2 < q.ns) {  // every tap's two samples lie inside the record
 #pragma unroll 4
-        for (int t = 0; t < q.ntx; ++t, row += tstride) {
+        for (int t = 0; t < q.ntx; ++t) {
           int i;
           float f;
-          das_tap(utx_s[t * DAS_THREADS + threadIdx.x], ur, i, f);
-          float a, b;
-          if ((unsigned)i < (unsigned)(q.ns - 1)) {  // both samples inside the record
-            a = __ldg(&row[i]);
-            b = __ldg(&row[i + 1]);
-          } else {
-            a = (i >= 0 && i < q.ns) ? __ldg(&row[i]) : 0.0f;
-            b = (i + 1 >= 0 && i + 1 < q.ns) ? __ldg(&row[i + 1]) : 0.0f;
-          }
-          s += fmaf(f, b - a, a);
+          das_tap(utx_s[t * DAS_PX + px], b, i, f);
+          const float v0 = __ldg(&rf[i]), v1 = __ldg(&rf[i + 1]);
+          s += fmaf(f, v1 - v0, v0);
         }
-        acc = fmaf(apod_w(q, im, x.hi, z.hi, e), s, acc);
+      } else {
+        for (int t = 0; t < q.ntx; ++t) {
+          int i;
+          float f;
+          das_tap(utx_s[t * DAS_PX + px], b, i, f);
+          const float* row = rf + (size_t)t * tstride + (size_t)e * q.ns;
+          i -= t * tstride + e * q.ns;
+          const float v0 = (i >= 0 && i < q.ns) ? __ldg(&row[i]) : 0.0f;
+          const float v1 = (i + 1 >= 0 && i + 1 < q.ns) ? __ldg(&row[i + 1]) : 0.0f;
+          s += fmaf(f, v1 - v0, v0);
+        }
       }
-      irf[p] = acc;
+      sb[(e - e0) * DAS_PX] = s;
+      if (dynamic) wb[(e - e0) * DAS_PX] = apod_w(q, im, x.hi, z.hi, e);
     }
+    __syncthreads();  // the other buffer is written next; this one again only after the next barrier
+    if (es == 0)
+      for (int e = e0; e < e1; ++e)
+        acc = fmaf(dynamic ? wb[(e - e0) * DAS_PX] : w_s[e], sb[(e - e0) * DAS_PX], acc);
   }
+  if (es == 0 && valid) irf[(size_t)l * im.nd + d] = acc;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -281,7 +357,7 @@ __global__ void __launch_bounds__(DT_THREADS) k_das_tma(Acq q, Img im, const flo
     }
     float2 ur[DT_PX];
 #pragma unroll
-    for (int p = 0; p < DT_PX; ++p) ur[p] = das_split(das_urx(q, g, x[p], z[p], e));
+    for (int p = 0; p < DT_PX; ++p) ur[p] = das_split(das_urx(das_rx(g, x[p], z[p]), das_elem(q, g, e)));
     float se[DT_PX];
 #pragma unroll
     for (int p = 0; p < DT_PX; ++p) se[p] = 0.0f;
@@ -418,7 +494,7 @@ __global__ void __launch_bounds__(DAS_THREADS) k_das_adj(Acq q, Img im, const fl
     const float gv = valid ? gi[p] : 0.0f;
     if (gv != 0.0f) {
       for (int e = 0; e < q.ne; ++e) {
-        const float2 ur = das_split(das_urx(q, g, x, z, e));
+        const float2 ur = das_split(das_urx(das_rx(g, x, z), das_elem(q, g, e)));
         const long long W = das_adj_fixed64(ldexpf(apod_w(q, im, x.hi, z.hi, e) * gv, kexp));
         for (int t = 0; t < q.ntx; ++t) {
           int i;
@@ -504,7 +580,7 @@ __global__ void __launch_bounds__(DJ_THREADS) k_das_adj_tile(Acq q, Img im, cons
     if (e + 1 < q.ne) dj_windows(q, im, l0, l1, d0, d1, e + 1, win_s + ((e + 1) & 1) * ntx, lane, warp);
     const long long W = gv != 0.0f ? das_adj_fixed64(ldexpf(apod_w(q, im, x.hi, z.hi, e) * gv, kexp)) : 0ll;
     if (W != 0ll) {
-      const float2 ur = das_split(das_urx(q, g, x, z, e));
+      const float2 ur = das_split(das_urx(das_rx(g, x, z), das_elem(q, g, e)));
 #pragma unroll 4
       for (int t = 0; t < ntx; ++t) {
         int i;
@@ -850,7 +926,7 @@ __global__ void __launch_bounds__(DA_THREADS) k_das_acq(Acq q, Img im, const flo
   float c0 = 0.0f, cp = 0.0f;  // sum slope u; sum slope du/dp
   if (gp != 0.0f) {
     for (int e = 0; e < q.ne; ++e) {
-      const float2 ur = das_split(das_urx(q, g, x, z, e));
+      const float2 ur = das_split(das_urx(das_rx(g, x, z), das_elem(q, g, e)));
       float dwp;
       const float w = apod_w(q, im, x.hi, z.hi, e, &dwp);
       const float ce = (float)e - hn;
@@ -886,14 +962,15 @@ __global__ void __launch_bounds__(DA_THREADS) k_das_acq(Acq q, Img im, const flo
 }
 
 // ------------------------------------------------------------------------------------------
-void launch_das(const Acq& q, const Img& im, const float* rf, float* irf, int grid, cudaStream_t st, int* status) {
+void launch_das(const Acq& q, const Img& im, const float* rf, float* irf, cudaStream_t st, int* status) {
   if (status && q.ne * q.ntx <= DT_MAX_WINDOWS && das_tma_smem(q) <= (size_t)DT_SMEM_MAX &&
       ((uintptr_t)rf & 15u) == 0) {
     const int tiles = ((im.nl + DT_LINES - 1) / DT_LINES) * ((im.nd + DT_DEPTHS - 1) / DT_DEPTHS);
     k_das_tma<<<tiles, DT_THREADS, das_tma_smem(q), st>>>(q, im, rf, irf, status);
     return;
   }
-  k_das<<<grid, DAS_THREADS, sizeof(float2) * DAS_THREADS * q.ntx, st>>>(q, im, rf, irf);
+  const int tiles = ((im.nl + DAS_TL - 1) / DAS_TL) * ((im.nd + DAS_TD - 1) / DAS_TD);
+  k_das<<<tiles, DAS_THREADS, das_smem(q.ne, q.ntx, im.fnum > 0.0f), st>>>(q, im, rf, irf);
 }
 int das_acq_blocks(const Img& im) { return (im.nl * im.nd + DA_THREADS - 1) / DA_THREADS; }
 void launch_das_acq(const Acq& q, const Img& im, const float* rf, const float* gi, float* part, cudaStream_t st) {
@@ -993,7 +1070,7 @@ cudaError_t image_set_attrs(int nd) {
   cudaError_t e0 = cudaFuncSetAttribute(k_envlog_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSED_SMEM_MAX);
   if (e0 != cudaSuccess) return e0;
   cudaError_t e = cudaFuncSetAttribute(k_das, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(float2) * DAS_THREADS * MAX_TX));
+                                       (int)das_smem(MAX_ELEM, MAX_TX, true));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_das_adj, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)(sizeof(float2) * DAS_THREADS * MAX_TX));

@@ -6,7 +6,7 @@
 namespace usrt {
 
 // DAS; with a device status word the TMA-staged kernel is used when the shape allows
-void launch_das(const Acq& q, const Img& im, const float* rf, float* irf, int grid, cudaStream_t st,
+void launch_das(const Acq& q, const Img& im, const float* rf, float* irf, cudaStream_t st,
                 int* status = nullptr);
 // transposed DAS, deterministic (64-bit fixed-point accumulation): acc is scratch of
 // ntx * ne * ns words, maxbits one word
