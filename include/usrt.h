@@ -195,7 +195,7 @@ void us_set_envlog_fused(int enable);
 
 /* Transposed DAS kernels, process-wide: enable != 0 (the default) uses the tiled kernel
  * (per-tile sample windows in shared memory, one global atomic per window entry) whenever
- * n_tx <= 32; 0 always takes the untiled kernel (one global atomic per tap).  Both give the
+ * n_tx <= 36; 0 always takes the untiled kernel (one global atomic per tap).  Both give the
  * same bits (the same fixed-point contributions).  Applies to us_das_adjoint, us_bmode_vjp and
  * us_adjoint; meant for tests of the second path. */
 void us_set_das_adj_tiled(int enable);

@@ -1,7 +1,9 @@
 // Image formation and its adjoint: delay-and-sum (Eq. das) and its transpose (Eq.
 // das_adjoint), the Hilbert envelope along depth, log compression with the dynamic-range clip
 // (Sec. 2.3.4), the l1/l2 loss (Eq. weighted_l1_l2_loss) and the envelope/log VJP.
+#include <algorithm>
 #include <atomic>
+#include <cmath>
 
 #include "image.cuh"
 
@@ -442,32 +444,33 @@ __device__ __forceinline__ int das_adj_kexp(int npx, unsigned int maxbits) {
 // already); 1.5 2^23 added with rounding toward -inf gives floor(v / 2^22) in the float's low
 // mantissa bits; the remainder is an exact subtraction.
 constexpr int DAS_ADJ_LO_BITS = 22;
-__device__ __forceinline__ void das_adj_fixed(float v, int& hi, uint32_t& lo) {
+__device__ __forceinline__ void das_adj_fixed(float v, int& hi, int& lo) {
   const float c = copysignf(8388608.0f, v);
   const float vr = fabsf(v) < 8388608.0f ? __fsub_rn(__fadd_rn(v, c), c) : v;
   const float h = __fadd_rd(vr * (1.0f / 4194304.0f), 12582912.0f);  // 1.5 2^23 + floor(vr / 2^22)
   hi = __float_as_int(h) - 0x4B400000;
   const float hf = __fsub_rn(h, 12582912.0f);
   const float lf = __fsub_rn(vr, hf * 4194304.0f);  // in [0, 2^22), exact
-  lo = __float_as_uint(__fadd_rn(lf, 8388608.0f)) - 0x4B000000u;
+  lo = __float_as_int(__fadd_rn(lf, 8388608.0f)) - 0x4B000000;
 }
-__device__ __forceinline__ long long das_adj_fixed64(float v) {
-  int hi;
-  uint32_t lo;
-  das_adj_fixed(v, hi, lo);
+// v 2^k (|v 2^k| < 2^43) without the range checks of ldexpf: two factors, each a normal float
+__device__ __forceinline__ float das_adj_scaled(float v, int k) {
+  const int a = k / 2, b = k - a;
+  return v * __int_as_float((127 + a) << 23) * __int_as_float((127 + b) << 23);
+}
+// the two samples' shares of W = wh 2^22 + wl at interpolation fraction f in [0, 1): 1 + f
+// rounded to the float grid of [1, 2) puts F = round(f 2^23) in the mantissa; the second
+// sample's share is s1 = floor(W F / 2^23) = h1 2^22 + l1 with l1 in [0, 2^22), cut out of the
+// 64-bit product; the first's is W - s1, word by word (its low word may be negative)
+__device__ __forceinline__ void das_adj_second(long long W, float f, int& h1, int& l1) {
+  const uint32_t F = (uint32_t)(__float_as_int(__fadd_rn(1.0f, f)) - 0x3F800000);
+  const unsigned long long lo = (unsigned long long)(uint32_t)W * F;
+  const int ph = (int)(W >> 32) * (int)F + (int)(lo >> 32);
+  h1 = ph >> (DAS_ADJ_LO_BITS + DAS_ADJ_F_BITS - 32);
+  l1 = (int)(__funnelshift_r((uint32_t)lo, (uint32_t)ph, DAS_ADJ_F_BITS) & ((1u << DAS_ADJ_LO_BITS) - 1u));
+}
+__device__ __forceinline__ long long das_adj_join(int hi, int lo) {
   return (long long)hi * (1ll << DAS_ADJ_LO_BITS) + (long long)lo;
-}
-// the two samples' shares of W at interpolation fraction f in [0, 1): 1 + f rounded to the
-// float grid of [1, 2) puts F = round(f 2^23) in the mantissa; s0 + s1 = W exactly
-__device__ __forceinline__ void das_adj_shares(long long W, float f, long long& s0, long long& s1) {
-  const long long F = (long long)(__float_as_int(__fadd_rn(1.0f, f)) - 0x3F800000);
-  s1 = (W * F) >> DAS_ADJ_F_BITS;  // arithmetic shift: floor
-  s0 = W - s1;
-}
-// a share as the tiled kernel's two words: hi 2^22 + lo, lo in [0, 2^22)
-__device__ __forceinline__ void das_adj_words(long long v, int& hi, uint32_t& lo) {
-  hi = (int)(v >> DAS_ADJ_LO_BITS);
-  lo = (uint32_t)v & ((1u << DAS_ADJ_LO_BITS) - 1u);
 }
 __global__ void k_das_adj_finish(const unsigned long long* __restrict__ acc, long long n, int npx,
                                  const unsigned int* maxbits, float* grf) {
@@ -491,19 +494,22 @@ __global__ void __launch_bounds__(DAS_THREADS) k_das_adj(Acq q, Img im, const fl
     const int l = valid ? p / im.nd : 0, d = valid ? p - l * im.nd : 0;
     const ff x = grid_coord(im.x0, im.x1, l, im.nl), z = grid_coord(im.z0, im.z1, d, im.nd);
     for (int t = 0; t < q.ntx; ++t) utx_s[t * DAS_THREADS + threadIdx.x] = das_split(das_utx(q, g, x, z, t));
-    const float gv = valid ? gi[p] : 0.0f;
+    const float gv = valid ? das_adj_scaled(gi[p], kexp) : 0.0f;
     if (gv != 0.0f) {
       for (int e = 0; e < q.ne; ++e) {
         const float2 ur = das_split(das_urx(das_rx(g, x, z), das_elem(q, g, e)));
-        const long long W = das_adj_fixed64(ldexpf(apod_w(q, im, x.hi, z.hi, e) * gv, kexp));
+        int wh, wl;
+        das_adj_fixed(apod_w(q, im, x.hi, z.hi, e) * gv, wh, wl);
+        const long long W = das_adj_join(wh, wl);
         for (int t = 0; t < q.ntx; ++t) {
           int i;
           float f;
           das_tap(utx_s[t * DAS_THREADS + threadIdx.x], ur, i, f);
-          long long s0, s1;
-          das_adj_shares(W, f, s0, s1);
+          int h1, l1;
+          das_adj_second(W, f, h1, l1);
+          const long long s1 = das_adj_join(h1, l1);
           unsigned long long* row = acc + ((size_t)t * q.ne + e) * q.ns;
-          if (i >= 0 && i < q.ns) atomicAdd(&row[i], (unsigned long long)s0);
+          if (i >= 0 && i < q.ns) atomicAdd(&row[i], (unsigned long long)(W - s1));
           if (i + 1 >= 0 && i + 1 < q.ns) atomicAdd(&row[i + 1], (unsigned long long)s1);
         }
       }
@@ -512,51 +518,67 @@ __global__ void __launch_bounds__(DAS_THREADS) k_das_adj(Acq q, Img im, const fl
 }
 
 // Tiled transposed DAS.  A CTA owns a 16-line x 32-depth pixel tile (one pixel per thread; a
-// warp holds 32 consecutive depths of one line).  Element by element, the taps of all transmits
-// go into per-transmit sample windows in shared memory, the window of (e, t) being the samples
-// the tile's delays can reach (FP32 delays at the tile's corners, padded); then every nonzero
-// window entry goes to its row with one global atomic.  A window spans ~100-200 samples against
-// the tile's 1024 taps per (e, t), so the global atomics drop several-fold.  A tap outside its
-// window (an underestimated window, or one longer than DJ_WIN) goes to the row directly.
-// A window entry is two 32-bit words with native shared atomics: a share v (|v| <= |W| < 2^40)
-// splits into v >> 22 (signed, |.| <= 2^18) and its low 22 bits (unsigned); at most 512 pixels
-// add to one entry, so neither word can overflow (2^27 and 2^31), and the flush rebuilds
-// hi 2^22 + lo exactly.  The shares and their sums are those of k_das_adj, so the two kernels
-// give the same bits.
-constexpr int DJ_THREADS = 512, DJ_LINES = 16, DJ_DEPTHS = 32, DJ_WIN = 192;  // 256: +0.07 ms
-constexpr int DJ_SMEM_MAX = 200 * 1024;
+// warp holds 32 consecutive depths of one line, whose taps fall on different samples).  The
+// elements go in batches of up to DJ_COLS (element, transmit) columns: the taps of a batch go
+// into a sample window per column in shared memory, the samples the tile's delays can reach
+// (FP32 delays at the tile's corners, padded); then every nonzero window entry goes to its row
+// with one global atomic.  A window spans ~100-200 samples against the tile's 512 taps per
+// column, so the global atomics drop several-fold.  A tap outside its window (an
+// underestimated window, or one longer than `win`) goes to the row directly.
+// A window entry is two 32-bit words with native shared atomics, hi 2^22 + lo: a share's high word
+// is at most 2^18 in size, its low word below 2^22, and at most 512 pixels add to one entry, so
+// neither sum can overflow (2^27 and 2^31) and the flush rebuilds the exact total.  The shares
+// and their sums are those of k_das_adj, so the two kernels give the same bits.
+// Bound by instruction issue (75 %) and shared memory (four atomics per tap, two wavefronts each).
+// 128 elements, 256 x 1024 pixels: 16 transmits 1550 -> 1175 us, one transmit 410 -> 213 us (both
+// shares used to be split from 64-bit values and every weight rescaled, 78 instructions per tap;
+// every element had two barriers of its own; a tile was one block, 112 of them for 97 x 512 pixels).
+constexpr int DJ_THREADS = 512, DJ_LINES = 16, DJ_DEPTHS = 32;
+constexpr int DJ_COLS = 16;  // columns per batch (one element's transmits when those are more)
+constexpr int DJ_BLOCKS = 2432;  // 1216: 16 transmits +6 %, 11 on 97 x 512 pixels -5 %
+constexpr int DJ_SMEM_MAX = 226 * 1024;
+constexpr int DJ_MAX_TX = 36;                    // beyond, the untiled kernel
+constexpr int DJ_WIN_MIN = 128, DJ_WIN_MAX = 640;
 static_assert(DJ_DEPTHS == 32 && DJ_LINES == 16 && DJ_THREADS / 32 == DJ_LINES, "a warp is one line's 32 depths");
-static_assert(DAS_ADJ_V_BITS - DAS_ADJ_LO_BITS + 9 < 31 && DAS_ADJ_LO_BITS + 9 < 32,
+static_assert(DAS_ADJ_V_BITS - DAS_ADJ_LO_BITS + 9 < 31 && DAS_ADJ_LO_BITS + 9 <= 31,
               "the tile's 512 contributions per entry fit both words");
-__host__ __device__ constexpr size_t das_adj_tile_smem(int ntx) {
-  return (2 * sizeof(uint32_t) * DJ_WIN + sizeof(float2) * DJ_THREADS + 2 * sizeof(int2)) * (size_t)ntx;
+__host__ __device__ constexpr int das_adj_batch(int ntx) { return ntx >= DJ_COLS ? 1 : DJ_COLS / ntx; }
+__host__ __device__ constexpr size_t das_adj_tile_smem(int ne, int ntx, int win) {
+  return (2 * sizeof(int) * win + 2 * sizeof(int2)) * (size_t)(das_adj_batch(ntx) * ntx) +
+         sizeof(float2) * ((size_t)DJ_THREADS * ntx + ne) + sizeof(float) * ne;
 }
-// windows of element e for all transmits: warp w takes transmits w, w + 16, ...; its lanes
-// evaluate the 32 corner delays (16 lines x the two depth ends) and reduce them
-__device__ __forceinline__ void dj_windows(const Acq& q, const Img& im, int l0, int l1, int d0, int d1, int e,
-                                           int2* out, int lane, int warp) {
-  for (int t = warp; t < q.ntx; t += DJ_THREADS / 32) {  // warp-uniform
-    const float u = das_delay_f32(q, im, min(l0 + (lane & 15), l1), (lane & 16) ? d1 : d0, e, t);
-    float lo = u, hi = u;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lo = fminf(lo, __shfl_xor_sync(0xFFFFFFFFu, lo, o));
-      hi = fmaxf(hi, __shfl_xor_sync(0xFFFFFFFFu, hi, o));
-    }
-    if (lane == 0) out[t] = das_window_of(q.ns, lo, hi, DJ_WIN);
-  }
+static_assert(das_adj_tile_smem(MAX_ELEM, DJ_MAX_TX, 256) <= (size_t)DJ_SMEM_MAX, "the most transmits fit");
+// window length for an image: the samples a tile's delays can span (a depth step moves a delay by
+// at most its two-way time, a line step by 1 + |sin th| times its one-way time), as far as shared
+// memory allows.  A fixed 192 sent every tap of a coarse depth grid (97 x 512 pixels over 58 mm)
+// to the rows: 566 us against 224.
+static int das_adj_win(const Acq& q, const Img& im) {
+  double smax = 0.0;
+  for (int t = 0; t < q.ntx; ++t) smax = std::max(smax, (double)std::fabs(q.sin_tx[t]));
+  const double k = (double)q.fs / q.cbf;
+  const double dz = im.nd > 1 ? std::fabs((double)im.z1 - im.z0) / (im.nd - 1) : 0.0;
+  const double dx = im.nl > 1 ? std::fabs((double)im.x1 - im.x0) / (im.nl - 1) : 0.0;
+  const double span = k * (2.0 * (DJ_DEPTHS - 1) * dz + (1.0 + smax) * (DJ_LINES - 1) * dx) + 12.0;
+  int win = span < DJ_WIN_MAX ? std::max(DJ_WIN_MIN, ((int)span + 31) / 32 * 32) : DJ_WIN_MAX;
+  while (win > DJ_WIN_MIN && das_adj_tile_smem(q.ne, q.ntx, win) > (size_t)DJ_SMEM_MAX) win -= 32;
+  return win;
 }
-__global__ void __launch_bounds__(DJ_THREADS) k_das_adj_tile(Acq q, Img im, const float* __restrict__ gi,
+__global__ void __launch_bounds__(DJ_THREADS) k_das_adj_tile(Acq q, Img im, int win, const float* __restrict__ gi,
                                                              unsigned long long* acc, const unsigned int* maxbits) {
   extern __shared__ __align__(16) unsigned char dj_sm[];
-  const int ntx = q.ntx;
-  int* hi_s = reinterpret_cast<int*>(dj_sm);                                   // [ntx][DJ_WIN]
-  uint32_t* lo_s = reinterpret_cast<uint32_t*>(hi_s + (size_t)ntx * DJ_WIN);   // [ntx][DJ_WIN]
-  float2* utx_s = reinterpret_cast<float2*>(lo_s + (size_t)ntx * DJ_WIN);      // [ntx][DJ_THREADS]
-  int2* win_s = reinterpret_cast<int2*>(utx_s + (size_t)ntx * DJ_THREADS);     // [2][ntx]
+  const int ntx = q.ntx, batch = das_adj_batch(ntx), ncol = batch * ntx;
+  int* hi_s = reinterpret_cast<int*>(dj_sm);                                // [ncol][win]
+  int* lo_s = hi_s + ncol * win;                                         // [ncol][win]
+  float2* utx_s = reinterpret_cast<float2*>(lo_s + ncol * win);          // [ntx][DJ_THREADS]
+  int2* win_s = reinterpret_cast<int2*>(utx_s + (size_t)ntx * DJ_THREADS);  // [2][ncol]
+  float2* xe_s = reinterpret_cast<float2*>(win_s + 2 * ncol);               // [ne] element positions (float-float)
+  float* w_s = reinterpret_cast<float*>(xe_s + q.ne);                       // [ne] Hann weights
   const unsigned int mb = *maxbits;
   if (mb >= F32_INF_BITS) return;  // k_das_adj_finish writes NaN
-  const int kexp = das_adj_kexp(im.nl * im.nd, mb);
+  // the tile's share of the elements: whole batches, split over gridDim.y blocks
+  const int per = ((q.ne + batch - 1) / batch + gridDim.y - 1) / gridDim.y * batch;
+  const int e_lo = blockIdx.y * per, e_hi = min(q.ne, e_lo + per);
+  if (e_lo >= e_hi) return;
   const int tiles_d = (im.nd + DJ_DEPTHS - 1) / DJ_DEPTHS;
   const int l0 = (blockIdx.x / tiles_d) * DJ_LINES, d0 = (blockIdx.x % tiles_d) * DJ_DEPTHS;
   const int l1 = min(l0 + DJ_LINES - 1, im.nl - 1), d1 = min(d0 + DJ_DEPTHS - 1, im.nd - 1);
@@ -566,56 +588,88 @@ __global__ void __launch_bounds__(DJ_THREADS) k_das_adj_tile(Acq q, Img im, cons
   const DasGeo g = das_geo(q);
   const ff x = grid_coord(im.x0, im.x1, valid ? l : l0, im.nl);
   const ff z = grid_coord(im.z0, im.z1, valid ? d : d0, im.nd);
-  const float gv = valid ? gi[(size_t)l * im.nd + d] : 0.0f;
+  const float gv = valid ? das_adj_scaled(gi[(size_t)l * im.nd + d], das_adj_kexp(im.nl * im.nd, mb)) : 0.0f;
   for (int t = 0; t < ntx; ++t) utx_s[t * DJ_THREADS + threadIdx.x] = das_split(das_utx(q, g, x, z, t));
-  for (int j = threadIdx.x; j < ntx * DJ_WIN; j += DJ_THREADS) {
-    hi_s[j] = 0;
-    lo_s[j] = 0u;
+  for (int j = threadIdx.x; j < 2 * ncol * win; j += DJ_THREADS) hi_s[j] = 0;  // both words
+  for (int e = e_lo + threadIdx.x; e < e_hi; e += DJ_THREADS) {
+    const ff xe = das_elem(q, g, e);
+    xe_s[e] = make_float2(xe.hi, xe.lo);
+    w_s[e] = hann_w(e, q.ne);
   }
-  dj_windows(q, im, l0, l1, d0, d1, 0, win_s, lane, warp);
+  const DasRx p = das_rx(g, x, z);
+  const bool dynamic = im.fnum > 0.0f;
+  // windows of a batch's columns: warp w takes columns w, w + 16, ...; its lanes hold the tile's 32
+  // corner positions (16 lines x the two depth ends).  A window is (first sample, entries the
+  // first share may go to): a tap is inside when its sample is less than that many past the
+  // first; nothing is inside an empty or overlong one.
+  const float cx = grid_coord(im.x0, im.x1, min(l0 + (lane & 15), l1), im.nl).hi;
+  const float cz = grid_coord(im.z0, im.z1, (lane & 16) ? d1 : d0, im.nd).hi;
+  const float kf = g.k.hi, hwf = g.half_w.hi;
+  auto windows = [&](int e0, int2* out) {
+    for (int c = warp; c < min(batch, e_hi - e0) * ntx; c += DJ_THREADS / 32) {  // warp-uniform
+      const int eb = c / ntx, t = c - eb * ntx;
+      const float dx = cx - (e0 + eb - 0.5f * (q.ne - 1)) * q.pitch;
+      const float u = (fmaf(cx, q.sin_tx[t], fmaf(cz, q.cos_tx[t], hwf * fabsf(q.sin_tx[t]))) + sqrtf(fmaf(dx, dx, cz * cz))) * kf;
+      const int lo = __reduce_min_sync(0xFFFFFFFFu, (int)floorf(u)), hi = __reduce_max_sync(0xFFFFFFFFu, (int)ceilf(u));
+      if (lane == 0) {
+        const int2 w = das_window_of(q.ns, lo, hi, win);
+        out[c] = make_int2(w.x, max(0, w.y - 1));
+      }
+    }
+  };
+  windows(e_lo, win_s);
   __syncthreads();
-  for (int e = 0; e < q.ne; ++e) {
-    const int2* wcur = win_s + (e & 1) * ntx;
-    // the other buffer was last read by the previous element's flush, before its barrier
-    if (e + 1 < q.ne) dj_windows(q, im, l0, l1, d0, d1, e + 1, win_s + ((e + 1) & 1) * ntx, lane, warp);
-    const long long W = gv != 0.0f ? das_adj_fixed64(ldexpf(apod_w(q, im, x.hi, z.hi, e) * gv, kexp)) : 0ll;
-    if (W != 0ll) {
-      const float2 ur = das_split(das_urx(das_rx(g, x, z), das_elem(q, g, e)));
-#pragma unroll 4
-      for (int t = 0; t < ntx; ++t) {
-        int i;
+  for (int e0 = e_lo, buf = 0; e0 < e_hi; e0 += batch, buf ^= 1) {
+    const int nb = min(batch, e_hi - e0);
+    const int2* wcur = win_s + buf * ncol;
+    // the other buffer was last read by the previous batch's flush, before its barrier
+    if (e0 + batch < e_hi) windows(e0 + batch, win_s + (buf ^ 1) * ncol);
+    for (int eb = 0; eb < nb; ++eb) {
+      const int e = e0 + eb;
+      int wh, wl;
+      das_adj_fixed((dynamic ? apod_w(q, im, x.hi, z.hi, e) : w_s[e]) * gv, wh, wl);
+      if ((wh | wl) == 0) continue;
+      const long long W = das_adj_join(wh, wl);
+      const float2 xe = xe_s[e];
+      const float2 ur = das_split(das_urx(p, ff{xe.x, xe.y}));
+      int* hc = hi_s + eb * ntx * win;
+      int* lc = lo_s + eb * ntx * win;
+      const int2* wc = wcur + eb * ntx;
+#pragma unroll 8
+      for (int t = 0; t < ntx; ++t, hc += win, lc += win) {
+        int i, h1, l1w;
         float f;
         das_tap(utx_s[t * DJ_THREADS + threadIdx.x], ur, i, f);
-        long long s0, s1;
-        das_adj_shares(W, f, s0, s1);
-        const int2 w = wcur[t];
-        const int rel = i - w.x;
-        if (w.y > 0 && rel >= 0 && rel + 1 < w.y) {
-          const int j = t * DJ_WIN + rel;
-          int h0, h1;
-          uint32_t o0, o1;
-          das_adj_words(s0, h0, o0);
-          das_adj_words(s1, h1, o1);
-          atomicAdd(&hi_s[j], h0);
-          atomicAdd(&lo_s[j], o0);
-          atomicAdd(&hi_s[j + 1], h1);
-          atomicAdd(&lo_s[j + 1], o1);
+        das_adj_second(W, f, h1, l1w);
+        const int2 w = wc[t];
+        const unsigned rel = (unsigned)i - (unsigned)w.x;
+        if (rel < (unsigned)w.y) {
+          atomicAdd(&hc[rel], wh - h1);
+          atomicAdd(&lc[rel], wl - l1w);
+          atomicAdd(&hc[rel + 1], h1);
+          atomicAdd(&lc[rel + 1], l1w);
         } else {
+          const long long s1 = das_adj_join(h1, l1w);
           unsigned long long* row = acc + ((size_t)t * q.ne + e) * q.ns;
-          if (i >= 0 && i < q.ns) atomicAdd(&row[i], (unsigned long long)s0);
+          if (i >= 0 && i < q.ns) atomicAdd(&row[i], (unsigned long long)(W - s1));
           if (i + 1 >= 0 && i + 1 < q.ns) atomicAdd(&row[i + 1], (unsigned long long)s1);
         }
       }
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < ntx * DJ_WIN; j += DJ_THREADS) {
-      const int t = j / DJ_WIN, r = j - t * DJ_WIN;
-      const int2 w = wcur[t];
-      if (r < w.y) {
-        const long long v = (long long)hi_s[j] * (1ll << DAS_ADJ_LO_BITS) + (long long)lo_s[j];
-        if (v) atomicAdd(acc + ((size_t)t * q.ne + e) * q.ns + w.x + r, (unsigned long long)v);
-        hi_s[j] = 0;  // both words, also when they cancel (v = 0 with hi = -lo / 2^22)
-        lo_s[j] = 0u;
+    for (int c = warp; c < nb * ntx; c += DJ_THREADS / 32) {  // a warp flushes a column
+      const int eb = c / ntx, t = c - eb * ntx;
+      const int2 w = wcur[c];
+      unsigned long long* row = acc + ((size_t)t * q.ne + e0 + eb) * q.ns + w.x;
+      for (int r = lane; r <= w.y; r += 32) {  // w.y + 1 entries; an empty window holds a zero
+        const int j = c * win + r;
+        const int h = hi_s[j], lo = lo_s[j];
+        if (h | lo) {
+          const long long v = das_adj_join(h, lo);
+          if (v) atomicAdd(&row[r], (unsigned long long)v);
+          hi_s[j] = 0;  // both words, also when they cancel (v = 0 with hi = -lo / 2^22)
+          lo_s[j] = 0;
+        }
       }
     }
     __syncthreads();
@@ -984,9 +1038,14 @@ void launch_das_adj(const Acq& q, const Img& im, const float* gi, float* grf, in
   cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * (size_t)n, st);
   cudaMemsetAsync(maxbits, 0, sizeof(unsigned int), st);
   k_das_adj_max<<<min(grid, (npx + 255) / 256), 256, 0, st>>>(gi, npx, maxbits);
-  if (das_adj_tile_smem(q.ntx) <= (size_t)DJ_SMEM_MAX && g_das_adj_tiled.load()) {
+  if (q.ntx <= DJ_MAX_TX && g_das_adj_tiled.load()) {
     const int tiles = ((im.nl + DJ_LINES - 1) / DJ_LINES) * ((im.nd + DJ_DEPTHS - 1) / DJ_DEPTHS);
-    k_das_adj_tile<<<tiles, DJ_THREADS, das_adj_tile_smem(q.ntx), st>>>(q, im, gi, acc, maxbits);
+    // a tile's elements over as many blocks as it takes to give the GPU DJ_BLOCKS of them
+    const int batches = (q.ne + das_adj_batch(q.ntx) - 1) / das_adj_batch(q.ntx);
+    const int split = max(1, min(batches, (DJ_BLOCKS + tiles - 1) / tiles));
+    const int win = das_adj_win(q, im);
+    k_das_adj_tile<<<dim3(tiles, split), DJ_THREADS, das_adj_tile_smem(q.ne, q.ntx, win), st>>>(q, im, win, gi, acc,
+                                                                                               maxbits);
   } else {
     k_das_adj<<<grid, DAS_THREADS, sizeof(float2) * DAS_THREADS * q.ntx, st>>>(q, im, gi, acc, maxbits);
   }

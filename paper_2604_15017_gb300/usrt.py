@@ -188,7 +188,7 @@ def set_envlog_fused(enable):
 
 
 def set_das_adj_tiled(enable):
-    """Process-wide: the tiled transposed-DAS kernel (True, default; n_tx <= 32) or always the
+    """Process-wide: the tiled transposed-DAS kernel (True, default; n_tx <= 36) or always the
     untiled one (False).  Same bits either way."""
     lib().us_set_das_adj_tiled(int(bool(enable)))
 

@@ -4,6 +4,7 @@ records that end inside the image (the checked taps), both apodisations.  Per pi
 the DAS of |RF| (the bound of test_gpu_parity.py)."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import oracle as O
 from paper_2604_15017_gb300 import phantoms as P
@@ -42,3 +43,31 @@ def test_das_matches_oracle_on_ragged_tiles(ctx, ne, ntx, ns, nl, nd, depth, f):
     bound = 2e-3 * O.das(q, im, np.abs(rf)) + 1e-6 * np.abs(ref).max()
     got = ctx.das(acq, img, dev(rf)).cpu().numpy()
     assert np.all(np.abs(got - ref) <= bound), np.max(np.abs(got - ref) - bound)
+
+
+@pytest.mark.parametrize("ne,ntx,ns,nl,nd,depth", [
+    (7, 3, 256, 5, 16, 4.0),       # fewer lines and depths than a tile
+    (100, 1, 4096, 33, 64, 60.0),  # coarse depths: windows of the largest size, some longer
+    (31, 15, 2048, 40, 256, 39.0),  # one element per batch but 15 columns
+    (101, 11, 3000, 97, 512, 57.0),
+    (24, 36, 1024, 20, 32, 15.0),  # the most transmits the tiled kernel takes, and one more
+    (24, 37, 1024, 20, 32, 15.0),
+])
+def test_transposed_das_tiled_equals_untiled(ctx, ne, ntx, ns, nl, nd, depth):
+    """The same fixed-point shares summed either way: the same bits, whatever window length, batch
+    of elements and split over blocks the sizes lead to."""
+    from paper_2604_15017_gb300 import usrt
+
+    angles = [7.0] if ntx == 1 else list(np.linspace(-20.0, 20.0, ntx))
+    acq = P.acquisition(ne, 0.3 * MM, ns, angles, 1, 1, 1540.0)
+    img = P.image(nl, nd, -0.16 * ne * MM, 0.15 * ne * MM, 0.0, depth * MM, f_number=1.5 if ntx == 15 else 0.0)
+    g = torch.Generator(device="cpu").manual_seed(ne)
+    gi = torch.randn(nl, nd, generator=g).cuda()
+    tiled = ctx.das_adjoint(acq, img, gi)
+    usrt.set_das_adj_tiled(False)
+    try:
+        plain = ctx.das_adjoint(acq, img, gi)
+    finally:
+        usrt.set_das_adj_tiled(True)
+    assert torch.equal(tiled, plain)
+    assert float(tiled.abs().max()) > 0.0
