@@ -29,7 +29,7 @@ enum Slot {
   W_ROW_CNT, W_ROW_OFF, W_ROW_CUR, W_BUCKET, W_SCRATCH, W_GTAB, W_IRF, W_ENV, W_KEY, W_PART, W_SCAL, W_GI,
   W_GRF, W_GPART, W_REC_CHUNK, W_PACK, W_NPACK, W_NEE_PATH, W_SEEDS, W_ACTIVE, W_ACT_CNT, W_RAY_KEY, W_RAY_CNT,
   W_RAY_OFF, W_RAY_CUR, W_JOBU_JOB, W_JOBU_JM, W_JOBU_PATH, W_GB, W_NEE_RES, W_NEE_XO, W_XING, W_PCLASS,
-  W_ACQ_PART, W_JOB_KEY, W_JOB_CNT, W_JOB_OFF, W_JOB_CUR, W_QA_SURF, W_KEEP, W_NEE_JX, W_NEE_JW, W_JOBU_JX,
+  W_ACQ_PART, W_JOB_KEY, W_JOB_CNT, W_JOB_OFF, W_JOB_CUR, W_QA_SURF, W_SCAT, W_NEE_JX, W_NEE_JW, W_JOBU_JX,
   W_JOBU_JW, W_QA_MIS, W_QB_MIS, W_SEEDV, W_DAS_ACC, W_DAS_MAX, W_COUNT
 };
 
@@ -99,6 +99,7 @@ struct us_ctx {
   Lane* L = nullptr;  // lane of the call in progress
   int num_sms = 148;
   int trav_per_sm = 4;   // blocks per SM of the traversal grid
+  int closest_per_sm = 4;  // resident blocks per SM of the joint closest-hit kernel
   int march_per_sm = 4;  // resident blocks per SM of the scatterer march
   int nee_per_sm = 4;    // resident blocks per SM of the secondary-ray kernel
   int* d_status = nullptr;    // device status word of kernels outside the transport (ST_* bits)
@@ -395,6 +396,8 @@ struct Queues {
   PathQ a, b;
 };
 
+constexpr uint32_t JOINT_MAX = 1u << 20;
+
 int alloc_queues(us_ctx* ctx, long long n, cudaStream_t st, Queues& Q) {
   CKS(ws(ctx, W_QA_PA, n, st, &Q.a.pa));
   CKS(ws(ctx, W_QA_WT, n, st, &Q.a.wt));
@@ -431,7 +434,7 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
   A.med = med;
   A.acq = q;
   CKS(ws(ctx, W_HITS, n, st, &A.hits));
-  CKS(ws(ctx, W_KEEP, n, st, &A.keep));
+  CKS(ws(ctx, W_SCAT, n, st, &A.scat));
   // secondary-ray jobs: the interaction kernel appends into `unsorted`, each round's jobs are
   // sorted into A.nee, which the secondary-ray kernel and the adjoint read
   const size_t jobs = (size_t)n * std::max(1, q.kmax);  // at most one job per path and round
@@ -524,9 +527,15 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
     A.qout = Q.a;
     if (sort_jobs) A.nee = unsorted;
     {
-      StageScope sc_(ctx, US_STAGE_TRAVERSE, sc->dev.n_scat > 0 ? 2 : 1, st);
-      launch_traverse(A, grid_of(ctx, ctx->trav_per_sm), st);
-      if (sc->dev.n_scat > 0) launch_march(A, grid_of(ctx, ctx->march_per_sm), st);
+      const bool scat = sc->dev.n_scat > 0;
+      A.joint = scat && n <= JOINT_MAX;
+      StageScope sc_(ctx, US_STAGE_TRAVERSE, scat && !A.joint ? 2 : 1, st);
+      if (A.joint) {
+        launch_closest(A, grid_of(ctx, ctx->closest_per_sm), st);
+      } else {
+        launch_traverse(A, grid_of(ctx, ctx->trav_per_sm), st);
+        if (scat) launch_march(A, grid_of(ctx, ctx->march_per_sm), st);
+      }
     }
     {
       StageScope sc_(ctx, US_STAGE_INTERACT, 1, st);
@@ -656,6 +665,7 @@ int us_create(us_ctx** out, int device, size_t mem_budget_bytes) {
   ctx->opts[US_OPT_NEE_STREAM] = 100;
   ctx->trav_per_sm = traverse_blocks_per_sm();
   ctx->march_per_sm = march_blocks_per_sm();
+  ctx->closest_per_sm = closest_blocks_per_sm();
   ctx->nee_per_sm = nee_blocks_per_sm();
   if (dev_alloc(ctx, (void**)&ctx->d_status, 256) != US_OK || cudaMemset(ctx->d_status, 0, 256) != cudaSuccess) {
     delete ctx;

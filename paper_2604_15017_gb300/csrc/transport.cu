@@ -122,20 +122,20 @@ __device__ __forceinline__ uint32_t warp_lanes(uint32_t n, uint32_t warps) {
 // of the BVH are fetched once per warp.  The scatterers are searched next by k_march below the
 // distance written here.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(TRAV_THREADS, 8) k_traverse(TransportArgs A) {
-  if (blockIdx.x == 0 && threadIdx.x == 0)  // secondary jobs of this round follow the previous rounds'
+// block `block` of `blocks` (`waves` waves of resident blocks)
+__device__ __forceinline__ void traverse_rays(const TransportArgs& A, uint32_t block, uint32_t blocks, uint32_t waves) {
+  if (block == 0 && threadIdx.x == 0)  // secondary jobs of this round follow the previous rounds'
     A.cnt->nee_off[A.k] = A.k ? A.cnt->nee_off[A.k - 1] + A.cnt->nee[A.k - 1] : 0u;
   const uint32_t n = *A.trav_n;  // the rest of the queue carries its surface hit
   // one wave of warps takes a small queue a few lanes each (warp_lanes); a larger one is walked
   // grid-stride, consecutive rays in one block
-  const uint32_t warps = gridDim.x * (TRAV_THREADS / 32) / 2;  // the grid is two waves
-  const uint32_t lanes = warp_lanes(n, warps);
+  const uint32_t lanes = warp_lanes(n, blocks * (TRAV_THREADS / 32) / waves);
   const uint32_t lane = threadIdx.x & 31u;
   const bool spread = lanes < 32u;
-  uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (spread) i = lane < lanes ? (blockIdx.x + gridDim.x * (threadIdx.x >> 5)) * lanes + lane : n;
+  uint32_t i = block * TRAV_THREADS + threadIdx.x;
+  if (spread) i = lane < lanes ? (block + blocks * (threadIdx.x >> 5)) * lanes + lane : n;
   bool overflow = false;
-  for (; i < n; i += spread ? n : gridDim.x * blockDim.x) {
+  for (; i < n; i += spread ? n : blocks * TRAV_THREADS) {
     const float4 pa = A.qin.pa[i];
     const float4 wt = A.qin.wt[i];
     const uint32_t prev = A.qin.meta[i].y;
@@ -145,6 +145,9 @@ __global__ void __launch_bounds__(TRAV_THREADS, 8) k_traverse(TransportArgs A) {
     A.hits[i] = make_float2(t, __uint_as_float(c == 0xFFFFFFFFu ? prim_code(CLS_NONE, 0) : c));
   }
   if (overflow) atomicOr(&A.cnt->status, ST_OVERFLOW);
+}
+__global__ void __launch_bounds__(TRAV_THREADS, 8) k_traverse(TransportArgs A) {
+  traverse_rays(A, blockIdx.x, gridDim.x, 2u);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -177,14 +180,19 @@ __global__ void __launch_bounds__(TRAV_THREADS, 8) k_traverse(TransportArgs A) {
 constexpr int MARCH_CHUNK = 32;
 constexpr int MARCH_REFILL_MIN = 4;
 
-__global__ void __launch_bounds__(MARCH_THREADS, 8) k_march(TransportArgs A) {
+// block `block` of `blocks` resident ones.  JOINT: rays before `unbounded`, whose surface hit is not
+// known yet, are searched to the end of the grid, and every ray's scat is written (t = 3e38:
+// none).  Else every ray is searched to its surface hit, and one that meets a scatterer first
+// gets its scat written and the flag set in its hit's code (writing every scat cost 2 % of the
+// march in the inclusion frame).
+template <bool JOINT>
+__device__ __forceinline__ void march_rays(const TransportArgs& A, uint32_t block, uint32_t blocks, uint32_t unbounded) {
   const SceneDev& S = A.S;
   const uint32_t n = A.cnt->live[A.k];
-  if (S.n_scat == 0 || n == 0) return;
   uint32_t* claim = &A.cnt->march[A.k];
   const unsigned lane = threadIdx.x & 31u;
   const unsigned below = (1u << lane) - 1u;
-  const uint32_t warps = gridDim.x * (MARCH_THREADS / 32);
+  const uint32_t warps = blocks * (MARCH_THREADS / 32);
   const uint32_t lanes = warp_lanes(n, warps);
   const uint32_t lane_mask = lanes >= 32u ? 0xFFFFFFFFu : (1u << lanes) - 1u;
   const uint32_t chunk = lanes >= 32u ? (uint32_t)MARCH_CHUNK : lanes;
@@ -198,8 +206,9 @@ __global__ void __launch_bounds__(MARCH_THREADS, 8) k_march(TransportArgs A) {
   float tnx = 0.0f, tny = 0.0f, tnz = 0.0f, kx = 0.0f, ky = 0.0f, kz = 0.0f;
   float dtx = 0.0f, dty = 0.0f, dtz = 0.0f, fx = 0.0f, fy = 0.0f, fz = 0.0f;
   int sx = 0, sy = 0, sz = 0, cell = 0;
-  float tbest = 0.0f, tend = 0.0f, t0hit = 0.0f;
-  uint32_t prev = 0u, cbest = 0u, code0 = 0u;
+  float tbest = 0.0f, tend = 0.0f;
+  uint32_t prev = 0u, cbest = 0u;
+  constexpr uint32_t NO_SCAT = 0u;  // before every code: a scatterer at the bound itself is none
   float4 slot_a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), slot_b = slot_a;  // the record to test next
   auto fetch = [&](int rec) {
     slot_a = __ldg(&S.cell_rec[2 * (size_t)rec]);
@@ -215,7 +224,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, 8) k_march(TransportArgs A) {
     }
   };
   // the first chunk of every warp is its own; the counter hands out the ones after those
-  uint32_t pool = min(n, (blockIdx.x + gridDim.x * (threadIdx.x >> 5)) * chunk);  // warp-uniform
+  uint32_t pool = min(n, (block + blocks * (threadIdx.x >> 5)) * chunk);  // warp-uniform
   uint32_t pool_end = min(n, pool + chunk);
   bool exhausted = pool >= n;  // warp-uniform
   while (true) {
@@ -243,12 +252,11 @@ __global__ void __launch_bounds__(MARCH_THREADS, 8) k_march(TransportArgs A) {
         ray = pool + rank;
         const float4 pa = A.qin.pa[ray];
         const float4 wt = A.qin.wt[ray];
-        const float2 hit = A.hits[ray];
+        tbest = JOINT && ray < unbounded ? 3.0e38f : A.hits[ray].x;
         o = xyz(pa);
         w = xyz(wt);
         prev = A.qin.meta[ray].y;
-        tbest = t0hit = hit.x;
-        cbest = code0 = __float_as_uint(hit.y);
+        cbest = NO_SCAT;
         const float ix = safe_inv(w.x), iy = safe_inv(w.y), iz = safe_inv(w.z);
         const float3 lo = S.glo;
         // the grid's slabs: t of the low faces and of the far ones
@@ -257,8 +265,9 @@ __global__ void __launch_bounds__(MARCH_THREADS, 8) k_march(TransportArgs A) {
         const float az = (lo.z - o.z) * iz, bz = (fmaf((float)nz, h, lo.z) - o.z) * iz;
         const float t0 = fmaxf(fmaxf(fminf(ax, bx), fminf(ay, by)), fmaxf(fminf(az, bz), 0.0f));
         const float t1 = fminf(fminf(fmaxf(ax, bx), fmaxf(ay, by)), fminf(fmaxf(az, bz), tbest));
-        if (t0 > t1) {
-          ray = 0xFFFFFFFFu;  // misses the grid before its surface hit: nothing to do
+        if (t0 > t1) {  // misses the grid before its surface hit
+          if (JOINT) A.scat[ray] = make_float2(3.0e38f, __uint_as_float(NO_SCAT));
+          ray = 0xFFFFFFFFu;
         } else {
           const float inv_h = 1.0f / h;
           const int cx = min(nx - 1, max(0, (int)floorf((fmaf(w.x, t0, o.x) - lo.x) * inv_h)));
@@ -316,9 +325,11 @@ __global__ void __launch_bounds__(MARCH_THREADS, 8) k_march(TransportArgs A) {
         tnz = fmaf(kz, dtz, fz);
       }
       if (!(t <= tbest && t < tend)) {  // no cell left to enter below tbest: done
-        if (cbest != code0) {  // a scatterer comes first; its pass-through carries the surface hit on
-          A.keep[ray] = make_float2(t0hit, __uint_as_float(code0));  // the hit this ray came with
-          A.hits[ray] = make_float2(tbest, __uint_as_float(cbest));
+        if (JOINT) {
+          A.scat[ray] = make_float2(cbest != NO_SCAT ? tbest : 3.0e38f, __uint_as_float(cbest));
+        } else if (cbest != NO_SCAT) {
+          A.scat[ray] = make_float2(tbest, __uint_as_float(cbest));
+          reinterpret_cast<uint8_t*>(&A.hits[ray])[7] = (uint8_t)(HIT_SCAT >> 24);  // codes have 22 bits
         }
         ray = 0xFFFFFFFFu;
         continue;
@@ -327,6 +338,22 @@ __global__ void __launch_bounds__(MARCH_THREADS, 8) k_march(TransportArgs A) {
     }
     fetch(rec);
   }
+}
+
+__global__ void __launch_bounds__(MARCH_THREADS, 8) k_march(TransportArgs A) {
+  if (A.cnt->live[A.k] > 0u) march_rays<false>(A, blockIdx.x, gridDim.x, 0u);
+}
+
+// Both searches of a round, side by side, for passes that do not keep the GPU full: the first half of the (resident)
+// blocks walk the BVH, the second half march the grid, without the surface bound for the rays
+// whose surface hit is not known yet.  Such a round lasts as long as the longest chain of
+// either search, so what the missing bound adds does not show, and the two chains overlap.
+__global__ void __launch_bounds__(TRAV_THREADS, 8) k_closest(TransportArgs A) {
+  const uint32_t half = gridDim.x / 2;
+  if (blockIdx.x < half)
+    traverse_rays(A, blockIdx.x, half, 1u);
+  else if (A.cnt->live[A.k] > 0u)
+    march_rays<true>(A, blockIdx.x - half, gridDim.x - half, *A.trav_n);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -354,13 +381,17 @@ __device__ __forceinline__ void interact_one(const TransportArgs& A, uint32_t i,
   const Acq& q = A.acq;
   const Media& med = A.med;
   const int K1 = q.kmax + 1;
-  const float2 h = A.hits[i];
+  float2 ks = A.hits[i];  // the surface hit
+  const float2 sc = A.scat[i];  // read with the slot's other words; what it holds counts below
+  const uint32_t kc = __float_as_uint(ks.y);
+  ks.y = __uint_as_float(kc & ~HIT_SCAT);
+  float2 h = ks;  // or a scatterer before it
+  if (A.joint ? hit_better(sc.x, __float_as_uint(sc.y), ks.x, kc) : (kc & HIT_SCAT) != 0u) h = sc;
   const uint32_t code = __float_as_uint(h.y);
   const uint32_t cls = code_cls(code);
   const uint4 meta = A.qin.meta[i];
   const float4 pa = A.qin.pa[i];  // read with the slot's other words, before the escape test
   const float4 wt = A.qin.wt[i];
-  const float2 ks = A.keep[i];  // used at scatterer events; read with the rest, not after the hit's class
   const long long path = meta.x;
   E.path = meta.x;
   uint32_t* rec = A.record ? &A.record[(size_t)(path - A.path_base) * K1 + A.k] : nullptr;
@@ -977,6 +1008,12 @@ void launch_generate(const TransportArgs& a, long long path0, uint32_t n, const 
 }
 void launch_traverse(const TransportArgs& a, int grid, cudaStream_t st) { k_traverse<<<grid, TRAV_THREADS, 0, st>>>(a); }
 void launch_march(const TransportArgs& a, int grid, cudaStream_t st) { k_march<<<grid, MARCH_THREADS, 0, st>>>(a); }
+void launch_closest(const TransportArgs& a, int grid, cudaStream_t st) { k_closest<<<grid, TRAV_THREADS, 0, st>>>(a); }
+int closest_blocks_per_sm() {
+  int b = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_closest, TRAV_THREADS, 0) != cudaSuccess || b < 1) b = 4;
+  return b;
+}
 int march_blocks_per_sm() {
   int b = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_march, MARCH_THREADS, 0) != cudaSuccess || b < 1) b = 4;

@@ -78,13 +78,18 @@ struct RaySort {
   uint32_t* cursor;     // [RAY_BUCKETS]
 };
 
+constexpr uint32_t HIT_SCAT = 0x80000000u;
+
 struct TransportArgs {
   SceneDev S;
   Media med;
   Acq acq;
   PathQ qin, qout;
-  float2* hits;       // (t, bits(code)) per queue slot
-  float2* keep;       // per queue slot: the surface hit a scatterer event replaced in hits
+  float2* hits;       // per queue slot: the surface hit (t, bits(code)); HIT_SCAT in the code: the
+                      // march found a scatterer before it
+  float2* scat;       // per queue slot: that scatterer's event
+  bool joint;         // both searches ran side by side (k_closest): scat holds the closest event of
+                      // every ray, before or past its surface hit, t = 3e38 when there is none
   const uint32_t* trav_n;  // rays of the sorted queue that need a surface query (the rest carry one)
   RaySort rk;         // keys and bucket counts of the rays appended to qout (the next round's sort)
   bool mis_on;        // secondary rays at rough events (the queues' mis fields are live)
@@ -118,6 +123,9 @@ void launch_traverse(const TransportArgs& a, int grid, cudaStream_t st);
 int traverse_blocks_per_sm();  // blocks per SM of the traversal grid
 constexpr int MARCH_THREADS = 128;
 void launch_march(const TransportArgs& a, int grid, cudaStream_t st);
+static_assert(MARCH_THREADS == TRAV_THREADS, "k_closest's blocks do either");
+void launch_closest(const TransportArgs& a, int grid, cudaStream_t st);  // both searches, resident grid
+int closest_blocks_per_sm();
 int march_blocks_per_sm();  // resident blocks per SM of the scatterer march (persistent grid)
 void launch_interact(const TransportArgs& a, int grid, cudaStream_t st);
 constexpr int NEE_THREADS = 128;
