@@ -30,7 +30,7 @@ enum Slot {
   W_GRF, W_GPART, W_REC_CHUNK, W_PACK, W_NPACK, W_NEE_PATH, W_SEEDS, W_ACTIVE, W_ACT_CNT, W_RAY_KEY, W_RAY_CNT,
   W_RAY_OFF, W_RAY_CUR, W_JOBU_JOB, W_JOBU_JM, W_JOBU_PATH, W_GB, W_NEE_RES, W_NEE_XO, W_XING, W_PCLASS,
   W_ACQ_PART, W_JOB_KEY, W_JOB_CNT, W_JOB_OFF, W_JOB_CUR, W_QA_SURF, W_SCAT, W_NEE_JX, W_NEE_JW, W_JOBU_JX,
-  W_JOBU_JW, W_QA_MIS, W_QB_MIS, W_SEEDV, W_DAS_ACC, W_DAS_MAX, W_COUNT
+  W_JOBU_JW, W_QB_SURF, W_QA_MIS, W_QB_MIS, W_SEEDV, W_DAS_ACC, W_DAS_MAX, W_COUNT
 };
 
 struct SceneGPU {
@@ -396,7 +396,17 @@ struct Queues {
   PathQ a, b;
 };
 
-constexpr uint32_t JOINT_MAX = 1u << 20;
+// A pass of at most SMALL_PASS paths does not keep the GPU full: its rounds last as long as their
+// longest chains.  It searches surfaces and scatterers side by side (k_closest) and leaves out
+// the coherence sorts of the rays and of the secondary-ray jobs, whose launches cost more than
+// the coherence gives.  Forward passes, two bounded sorted searches against one joint unsorted
+// one: 1e5 paths (12 regions, 1e5 scatterers) 1.23 -> 1.08 ms per iteration for the sorts alone,
+// 1.0M 2.39 -> 2.25 ms, 1.4M 3.15 -> 2.78, 2.0M 3.73 -> 3.62, 3.1M 4.71 -> 4.97, 4.1M 5.77 -> 6.36;
+// 3 regions and 3000 scatterers, 2.0M 1.43 -> 1.26 ms, 4.1M 1.94 -> 1.93.
+constexpr uint32_t SMALL_PASS = 1u << 21;
+// scenes without scatterers and with at most this many triangles need no sort at any size (every
+// ray visits the same few nodes): two layers, 12 triangles, 6.4e5 paths 362 -> 268 us
+constexpr int UNSORTED_TRIS = 64;
 
 int alloc_queues(us_ctx* ctx, long long n, cudaStream_t st, Queues& Q) {
   CKS(ws(ctx, W_QA_PA, n, st, &Q.a.pa));
@@ -453,8 +463,10 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
     CKS(ws(ctx, W_QA_MIS, n, st, &Q.a.mis));
     CKS(ws(ctx, W_QB_MIS, n, st, &Q.b.mis));
   }
+  A.sort = !(n <= SMALL_PASS || (sc->dev.n_scat == 0 && sc->dev.n_tris <= UNSORTED_TRIS));
+  if (!A.sort) CKS(ws(ctx, W_QB_SURF, n, st, &Q.b.surf));
   NeeQ sorted = A.nee, unsorted;
-  const bool sort_jobs = any_jobs;
+  const bool sort_jobs = any_jobs && A.sort;
   if (sort_jobs) {
     CKS(ws(ctx, W_JOBU_JOB, jobs, st, &unsorted.job));
     CKS(ws(ctx, W_JOBU_JM, jobs, st, &unsorted.jm));
@@ -512,23 +524,26 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
   // Q.a: rays as the interaction kernel appends them; Q.b: coherence-sorted (the emission
   // writes there directly)
   A.qout = Q.b;
-  {
+  if (!A.sort) {
+    StageScope sc_(ctx, US_STAGE_GENERATE, 1, st);
+    launch_generate_unsorted(A, path0, n, grid_of(ctx, 8), st);
+  } else {
     StageScope sc_(ctx, US_STAGE_GENERATE, 3, st);
     CK(cudaMemsetAsync(rs.cnt, 0, sizeof(uint32_t) * RAY_BUCKETS, st));
     launch_generate(A, path0, n, rs, grid_of(ctx, 2), st);
   }
   for (int k = 0; k <= q.kmax; ++k) {
     A.k = k;
-    if (k > 0) {
+    if (k > 0 && A.sort) {
       StageScope sc_(ctx, US_STAGE_RAY_SORT, 2, st);
       launch_ray_sort(A, Q.a, Q.b, rs, grid_of(ctx, 2), st);
     }
-    A.qin = Q.b;
-    A.qout = Q.a;
+    A.qin = A.sort || !(k & 1) ? Q.b : Q.a;
+    A.qout = A.sort || !(k & 1) ? Q.a : Q.b;
     if (sort_jobs) A.nee = unsorted;
     {
       const bool scat = sc->dev.n_scat > 0;
-      A.joint = scat && n <= JOINT_MAX;
+      A.joint = scat && n <= SMALL_PASS;
       StageScope sc_(ctx, US_STAGE_TRAVERSE, scat && !A.joint ? 2 : 1, st);
       if (A.joint) {
         launch_closest(A, grid_of(ctx, ctx->closest_per_sm), st);
@@ -539,7 +554,8 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
     }
     {
       StageScope sc_(ctx, US_STAGE_INTERACT, 1, st);
-      CK(cudaMemsetAsync(rs.cnt, 0, sizeof(uint32_t) * RAY_BUCKETS, st));  // this round's sort has scanned them
+      if (A.sort)  // this round's sort has scanned them
+        CK(cudaMemsetAsync(rs.cnt, 0, sizeof(uint32_t) * RAY_BUCKETS, st));
       launch_interact(A, grid_of(ctx, 8), st);
     }
     // the round's secondary rays (job sort, then the kernel): on the second stream from here

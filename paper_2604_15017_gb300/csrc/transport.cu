@@ -82,6 +82,20 @@ __device__ __forceinline__ void emit_path(const Acq& q, long long path, float3& 
   o0 = f3(xe + (u0 - 0.5f) * q.pitch, (u1 - 0.5f) * q.hel, 0.0f);
   w0 = f3(r * cp, r * sp, sqrtf(1.0f - u2));
 }
+// an unsorted pass's emission: path path0 + i in slot i
+__global__ void __launch_bounds__(256) k_generate(TransportArgs A, long long path0, uint32_t n) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    float3 o0, w0;
+    float tau0;
+    emit_path(A.acq, path0 + i, o0, w0, tau0);
+    A.qout.pa[i] = make_float4(o0.x, o0.y, o0.z, 3.14159265358979f / A.acq.nr);
+    A.qout.wt[i] = make_float4(w0.x, w0.y, w0.z, tau0);
+    A.qout.meta[i] = make_uint4((uint32_t)(path0 + i), 0xFFFFFFFFu, 0u, __float_as_uint(0.0f));
+    A.qout.surf[i] = make_float2(-1.0f, 0.0f);
+    if (A.mis_on) A.qout.mis[i] = make_float2(0.0f, 0.0f);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) A.cnt->live[0] = n;
+}
 // The emitted rays go straight into coherence-sorted order: this pass counts their sort keys
 // (they share few, all starting on the probe face, so the block counts in shared memory and adds
 // the nonzero counts once) and keeps each ray's key; k_generate_sorted emits them again, after
@@ -126,7 +140,8 @@ __device__ __forceinline__ uint32_t warp_lanes(uint32_t n, uint32_t warps) {
 __device__ __forceinline__ void traverse_rays(const TransportArgs& A, uint32_t block, uint32_t blocks, uint32_t waves) {
   if (block == 0 && threadIdx.x == 0)  // secondary jobs of this round follow the previous rounds'
     A.cnt->nee_off[A.k] = A.k ? A.cnt->nee_off[A.k - 1] + A.cnt->nee[A.k - 1] : 0u;
-  const uint32_t n = *A.trav_n;  // the rest of the queue carries its surface hit
+  // in a sorted queue the rays that carry their surface hit come last (and their hits are there)
+  const uint32_t n = A.sort ? *A.trav_n : A.cnt->live[A.k];
   // one wave of warps takes a small queue a few lanes each (warp_lanes); a larger one is walked
   // grid-stride, consecutive rays in one block
   const uint32_t lanes = warp_lanes(n, blocks * (TRAV_THREADS / 32) / waves);
@@ -136,6 +151,13 @@ __device__ __forceinline__ void traverse_rays(const TransportArgs& A, uint32_t b
   if (spread) i = lane < lanes ? (block + blocks * (threadIdx.x >> 5)) * lanes + lane : n;
   bool overflow = false;
   for (; i < n; i += spread ? n : blocks * TRAV_THREADS) {
+    if (!A.sort) {
+      const float2 sf = A.qin.surf[i];
+      if (sf.x >= 0.0f) {
+        A.hits[i] = sf;
+        continue;
+      }
+    }
     const float4 pa = A.qin.pa[i];
     const float4 wt = A.qin.wt[i];
     const uint32_t prev = A.qin.meta[i].y;
@@ -252,7 +274,12 @@ __device__ __forceinline__ void march_rays(const TransportArgs& A, uint32_t bloc
         ray = pool + rank;
         const float4 pa = A.qin.pa[ray];
         const float4 wt = A.qin.wt[ray];
-        tbest = JOINT && ray < unbounded ? 3.0e38f : A.hits[ray].x;
+        if (JOINT && !A.sort) {
+          tbest = A.qin.surf[ray].x;  // carried, or none
+          if (tbest < 0.0f) tbest = 3.0e38f;
+        } else {
+          tbest = JOINT && ray < unbounded ? 3.0e38f : A.hits[ray].x;
+        }
         o = xyz(pa);
         w = xyz(wt);
         prev = A.qin.meta[ray].y;
@@ -353,7 +380,7 @@ __global__ void __launch_bounds__(TRAV_THREADS, 8) k_closest(TransportArgs A) {
   if (blockIdx.x < half)
     traverse_rays(A, blockIdx.x, half, 1u);
   else if (A.cnt->live[A.k] > 0u)
-    march_rays<true>(A, blockIdx.x - half, gridDim.x - half, *A.trav_n);
+    march_rays<true>(A, blockIdx.x - half, gridDim.x - half, A.sort ? *A.trav_n : 0u);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -566,7 +593,7 @@ __global__ void __launch_bounds__(IA_THREADS, 3) k_interact(TransportArgs A) {
       A.qout.meta[o] = E.meta;
       A.qout.surf[o] = E.surf;
       if (A.mis_on) A.qout.mis[o] = E.mis;
-      ray_key_count(A.rk, o, xyz(E.pa), xyz(E.wt), E.surf.x >= 0.0f);
+      if (A.sort) ray_key_count(A.rk, o, xyz(E.pa), xyz(E.wt), E.surf.x >= 0.0f);
     }
     if (E.job) {
       const uint32_t slot = A.cnt->nee_off[A.k] + s_base[1] + s_pre[1][wid] + __popc(mj & below);
@@ -1005,6 +1032,9 @@ void launch_generate(const TransportArgs& a, long long path0, uint32_t n, const 
   k_generate_count<<<grid, GEN_THREADS, sizeof(uint32_t) * RAY_BUCKETS, st>>>(a, path0, n);
   launch_count_scan(rs.cnt, rs.off, rs.cursor, RAY_BUCKETS, st);
   k_generate_sorted<<<grid, RS_THREADS, scatter_smem(RAY_BUCKETS, RAY_CH), st>>>(a, path0, n, rs);
+}
+void launch_generate_unsorted(const TransportArgs& a, long long path0, uint32_t n, int grid, cudaStream_t st) {
+  k_generate<<<min((uint32_t)grid, (n + 255u) / 256u), 256, 0, st>>>(a, path0, n);
 }
 void launch_traverse(const TransportArgs& a, int grid, cudaStream_t st) { k_traverse<<<grid, TRAV_THREADS, 0, st>>>(a); }
 void launch_march(const TransportArgs& a, int grid, cudaStream_t st) { k_march<<<grid, MARCH_THREADS, 0, st>>>(a); }

@@ -90,6 +90,7 @@ struct TransportArgs {
   float2* scat;       // per queue slot: that scatterer's event
   bool joint;         // both searches ran side by side (k_closest): scat holds the closest event of
                       // every ray, before or past its surface hit, t = 3e38 when there is none
+  bool sort;          // the queues are coherence-sorted (else in the order their rays were appended)
   const uint32_t* trav_n;  // rays of the sorted queue that need a surface query (the rest carry one)
   RaySort rk;         // keys and bucket counts of the rays appended to qout (the next round's sort)
   bool mis_on;        // secondary rays at rough events (the queues' mis fields are live)
@@ -118,6 +119,8 @@ cudaError_t ray_sort_set_attrs();
 // counted into rs.cnt, zeroed by the caller, then scanned)
 void launch_generate(const TransportArgs& a, long long path0, uint32_t n, const RaySort& rs, int grid,
                      cudaStream_t st);
+// emission in path order, for a pass without the coherence sort
+void launch_generate_unsorted(const TransportArgs& a, long long path0, uint32_t n, int grid, cudaStream_t st);
 constexpr int TRAV_THREADS = 128;
 void launch_traverse(const TransportArgs& a, int grid, cudaStream_t st);
 int traverse_blocks_per_sm();  // blocks per SM of the traversal grid
