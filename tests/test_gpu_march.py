@@ -58,3 +58,37 @@ def test_grids_one_cell_thick(ctx, axis):
     w = no_triangles(P.slab_scatterers(n_rays=400, n_scat=3000))
     w["scat_pos"][:, axis] = [0.0, 0.0, 12 * MM][axis]  # a sheet of scatterers
     parity(ctx, w)
+
+
+@pytest.mark.parametrize("make", [
+    lambda: P.slab_scatterers(n_rays=33000, n_scat=4000),
+    lambda: P.with_roughness(P.hollow_cylinder(n_rays=33000), [0.0, 0.2, 0.0]),
+    lambda: P.inclusions(n_regions=3, n_scat=2000, n_rays=33000, angles_deg=[0.0], n_elem=64, n_samples=2048, n_lat=20,
+                         n_lon=40),
+    lambda: no_triangles(P.slab_scatterers(n_rays=33000, n_scat=4000)),
+    lambda: P.hollow_cylinder(n_rays=33000, n_scat=1),
+], ids=["slab", "rough", "inclusions", "scatterers", "surfaces"])
+def test_small_and_large_passes_decide_alike(ctx, make):
+    """A pass of more than 2^21 paths sorts its rays and searches surfaces before scatterers; one of
+    fewer searches both at once, unsorted.  Sub-apertures partition the full aperture's
+    realisation, so four small passes make the large one's records, word for word."""
+    w = make()
+    acq = w["acq"]
+    n = acq["n_elem"] * acq["n_rays"]
+    assert n > 1 << 21
+    sid = ctx.upload_workload(w)
+    ctx.forward(sid, w["theta"], acq, seed=5, keep_record=True)
+    full = ctx.record(0, n, acq["k_max"])
+    st = ctx.stats()
+    segments = arrivals = 0
+    for b in range(4):
+        part = dict(acq, tx_elem=16 * b, n_tx_elem=16)
+        ctx.forward(sid, w["theta"], part, seed=5, keep_record=True)
+        m = 16 * acq["n_rays"]
+        assert torch.equal(ctx.record(0, m, acq["k_max"]), full[b * m:(b + 1) * m])
+        s = ctx.stats()
+        assert s["status"] == 0
+        segments += s["segments"]
+        arrivals += s["arrivals"]
+    assert (segments, arrivals) == (st["segments"], st["arrivals"])
+    ctx.release_scene(sid)
