@@ -16,6 +16,7 @@ struct PulseP {
   // (cos, sin), and the Gaussian's ratio E(x + 1/fs) / E(x) is multiplied by
   // exp(-2 / (fs^2 sigma)) every sample
   float rot_c, rot_s, env_qq;
+  bool vec;  // the gathered rows are 16-byte aligned: four samples per read
 };
 
 struct AdjArgs {

@@ -365,6 +365,7 @@ int splat_geom(us_ctx* ctx, const Acq& q, float f0, SplatGeom& g, PulseP& P) {
   P.ns = q.ns;
   P.rot_c = (float)std::cos(2.0 * M_PI * (double)f0 / q.fs);
   P.rot_s = (float)std::sin(2.0 * M_PI * (double)f0 / q.fs);
+  P.vec = false;  // set where the gathered buffer is known
   P.env_qq = (float)std::exp(-2.0 / ((double)q.fs * q.fs * sig));
   return US_OK;
 }
@@ -1187,6 +1188,7 @@ int us_splat_adjoint(us_ctx* ctx, const us_acq_desc* acq, float f0, int64_t n, c
   if (n < 0 || (n && (!tx_dev || !e_dev || !tau_dev || !a_dev || !dL_drf_dev || !ga_dev || !gt_dev || !gf_dev)))
     return fail(ctx, US_ERR_ARG, "invalid arrival list");
   if (n) {
+    P.vec = aligned16(dL_drf_dev);
     StageScope sc_(ctx, US_STAGE_OTHER, 1, (cudaStream_t)stream);
     launch_splat_adjoint(q, P, tx_dev, e_dev, tau_dev, a_dev, n, dL_drf_dev, ga_dev, gt_dev, gf_dev, grid_of(ctx, 4),
                          (cudaStream_t)stream);
@@ -1219,6 +1221,7 @@ static int transport_vjp(us_ctx* ctx, uint64_t scene, const float* theta, const 
   A.med = med;
   A.acq = q;
   A.grf = dL_drf_dev;
+  A.pulse.vec = aligned16(dL_drf_dev);
   const int Ps = n_theta(med);
   A.P = Ps;
   A.acq_slot = -1;
