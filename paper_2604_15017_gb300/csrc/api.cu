@@ -27,7 +27,7 @@ struct Buf {
 enum Slot {
   W_QA_PA, W_QA_WT, W_QA_META, W_QB_PA, W_QB_WT, W_QB_META, W_HITS, W_NEE_JOB, W_NEE_JM, W_ARR, W_CNT,
   W_ROW_CNT, W_ROW_OFF, W_ROW_CUR, W_BUCKET, W_SCRATCH, W_GTAB, W_IRF, W_ENV, W_KEY, W_PART, W_SCAL, W_GI,
-  W_GRF, W_GPART, W_REC_CHUNK, W_PACK, W_NPACK, W_NEE_PATH, W_SEEDS, W_ACTIVE, W_ACT_CNT, W_RAY_KEY, W_RAY_CNT,
+  W_GRF, W_GPART, W_REC_CHUNK, W_NEE_PATH, W_SEEDS, W_ACTIVE, W_ACT_CNT, W_RAY_KEY, W_RAY_CNT,
   W_RAY_OFF, W_RAY_CUR, W_JOBU_JOB, W_JOBU_JM, W_JOBU_PATH, W_GB, W_NEE_RES, W_NEE_XO, W_XING, W_PCLASS,
   W_ACQ_PART, W_JOB_KEY, W_JOB_CNT, W_JOB_OFF, W_JOB_CUR, W_QA_SURF, W_SCAT, W_NEE_JX, W_NEE_JW, W_JOBU_JX,
   W_JOBU_JW, W_QB_SURF, W_QA_MIS, W_QB_MIS, W_SEEDV, W_DAS_ACC, W_DAS_MAX, W_COUNT
@@ -584,8 +584,9 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
   return US_OK;
 }
 
-int do_splat(us_ctx* ctx, const Acq& q, float f0, const Arrival* arr, const uint32_t* n_arr, uint32_t cap, float* rf,
-             cudaStream_t st) {
+// sort: launches the row bucketing of the arrivals (at most cap of them)
+template <class Sort>
+int do_splat(us_ctx* ctx, const Acq& q, float f0, size_t cap, float* rf, cudaStream_t st, Sort&& sort) {
   SplatGeom g;
   PulseP P;
   CKS(splat_geom(ctx, q, f0, g, P));
@@ -593,14 +594,14 @@ int do_splat(us_ctx* ctx, const Acq& q, float f0, const Arrival* arr, const uint
   CKS(ws(ctx, W_ROW_CNT, g.nrows, st, &w.row_cnt));
   CKS(ws(ctx, W_ROW_OFF, g.nrows + 1, st, &w.row_off));
   CKS(ws(ctx, W_ROW_CUR, g.nrows, st, &w.row_cursor));
-  CKS(ws(ctx, W_BUCKET, (size_t)cap + 1, st, &w.bucket));
-  CKS(ws(ctx, W_SCRATCH, (size_t)cap + 1, st, &w.scratch));
+  CKS(ws(ctx, W_BUCKET, cap + 1, st, &w.bucket));
+  CKS(ws(ctx, W_SCRATCH, cap + 1, st, &w.scratch));
   float* G;
   CKS(ws(ctx, W_GTAB, K_MOM * MAX_TAPS, st, &G));
   {
     StageScope sc_(ctx, US_STAGE_SPLAT_SORT, 4, st);
     launch_pulse_table(g, G, st);
-    launch_splat_sort(g, arr, n_arr, cap, w, grid_of(ctx, 4), st);
+    sort(g, w, grid_of(ctx, 4));
   }
   {
     StageScope sc_(ctx, US_STAGE_SPLAT_ROWS, 1, st);
@@ -953,7 +954,9 @@ int us_forward(us_ctx* ctx, uint64_t scene, const float* theta, const us_acq_des
     record = (uint32_t*)ctx->L->record.p;
   }
   CKS(run_transport(ctx, sc, med, q, 0, (uint32_t)n_paths, arr, cap, record, true, cnt, st));
-  CKS(do_splat(ctx, q, med.f0, arr, &cnt->n_arr, cap, rf_dev, st));
+  CKS(do_splat(ctx, q, med.f0, cap, rf_dev, st, [&](const SplatGeom& g, const SplatWork& w, int grid) {
+    launch_splat_sort(g, arr, &cnt->n_arr, cap, w, grid, st);
+  }));
   if (bmode_dev) CKS(do_bmode(ctx, q, im, rf_dev, bmode_dev, st));
   CK(cudaMemcpyAsync(ctx->L->h_cnt, cnt, sizeof(Counters), cudaMemcpyDeviceToHost, st));
   CK(cudaEventRecord(ctx->L->ev_stats, st));
@@ -1029,16 +1032,9 @@ int us_splat(us_ctx* ctx, const us_acq_desc* acq, float f0, int64_t n, const int
   if (n < 0 || n >= 0xFFFFFFF0ll || !rf_dev || !aligned16(rf_dev) || (n && (!tx_dev || !e_dev || !tau_dev || !a_dev)))
     return fail(ctx, US_ERR_ARG, "invalid arrival list");
   ctx->L->ikey.valid = false;  // rf_dev is rewritten
-  Arrival* arr;
-  uint32_t* n_out;
-  CKS(ws(ctx, W_PACK, (size_t)n + 1, st, &arr));
-  CKS(ws(ctx, W_NPACK, 1, st, &n_out));
-  CK(cudaMemsetAsync(n_out, 0, sizeof(uint32_t), st));
-  if (n) {
-    StageScope sc_(ctx, US_STAGE_OTHER, 1, st);
-    launch_pack_arrivals(tx_dev, e_dev, tau_dev, a_dev, n, q.ne, q.fs, arr, n_out, grid_of(ctx, 4), st);
-  }
-  return do_splat(ctx, q, f0, arr, n_out, (uint32_t)n + 1, rf_dev, st);
+  return do_splat(ctx, q, f0, (size_t)n, rf_dev, st, [&](const SplatGeom& g, const SplatWork& w, int grid) {
+    launch_splat_sort_list(g, tx_dev, e_dev, tau_dev, a_dev, (uint32_t)n, q.ne, q.fs, w, grid, st);
+  });
 }
 
 int us_das(us_ctx* ctx, const us_acq_desc* acq, const us_img_desc* img, const float* rf_dev, float* irf_dev,

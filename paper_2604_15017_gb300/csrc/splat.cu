@@ -8,11 +8,7 @@
 //      and finally the convolution RF[n] = sum_j sum_d G_j(d) M_j(n - d) with the table
 //        G_j(d) = g^(j)(d - 1/2) / j!,  g(x) = s(x / fs)
 //      (truncation after 8 moments: |delta| <= 1/2 sample gives < 1e-7 relative error).
-#include <cooperative_groups.h>
-
 #include "splat.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace usrt {
 
@@ -64,13 +60,55 @@ __global__ void k_pulse_table(SplatGeom g, float* G) {
 // ------------------------------------------------------------------------------------------
 // 1. bucket by row
 // ------------------------------------------------------------------------------------------
-__global__ void k_row_hist(const Arrival* arr, const uint32_t* n_arr, uint32_t cap, uint32_t* row_cnt, int nrows) {
+// Where the arrivals come from: the transport's packed list (its count on the device), or the
+// caller's four arrays, packed as they are read (a pass of its own that packed them, one atomic
+// per warp on one counter, took 200 us for 7.9M arrivals).  get() gives (row, tq, bits(a)), false
+// for an arrival outside the time range.
+struct PackedArrivals {
+  const Arrival* arr;
+  const uint32_t* n_arr;
+  uint32_t cap;
+  __device__ __forceinline__ uint32_t count() const { return min(*n_arr, cap); }
+  __device__ __forceinline__ bool row(uint32_t i, uint32_t& r) const {
+    r = arr[i].x;
+    return true;
+  }
+  __device__ __forceinline__ bool get(uint32_t i, uint32_t& r, uint2& v) const {
+    const Arrival A = arr[i];
+    r = A.x;
+    v = make_uint2(A.y, A.z);
+    return true;
+  }
+};
+struct ListedArrivals {
+  const int32_t *tx, *e;
+  const float *tau, *a;
+  uint32_t n;
+  int ne;
+  float fs;
+  __device__ __forceinline__ uint32_t count() const { return n; }
+  __device__ __forceinline__ bool row(uint32_t i, uint32_t& r) const {
+    r = (uint32_t)(__ldg(&tx[i]) * ne + __ldg(&e[i]));
+    return time_to_tq(__ldg(&tau[i]), 0.0f, fs) != 0xFFFFFFFFu;
+  }
+  __device__ __forceinline__ bool get(uint32_t i, uint32_t& r, uint2& v) const {
+    const uint32_t tq = time_to_tq(__ldg(&tau[i]), 0.0f, fs);
+    r = (uint32_t)(__ldg(&tx[i]) * ne + __ldg(&e[i]));
+    v = make_uint2(tq, __float_as_uint(__ldg(&a[i])));
+    return tq != 0xFFFFFFFFu;
+  }
+};
+template <class Src>
+__global__ void k_row_hist(Src src, uint32_t* row_cnt, int nrows) {
   extern __shared__ uint32_t h[];
+  const uint32_t n = src.count();
+  if (blockIdx.x * blockDim.x >= n) return;
   for (int r = threadIdx.x; r < nrows; r += blockDim.x) h[r] = 0;
   __syncthreads();
-  const uint32_t n = min(*n_arr, cap);
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    atomicAdd(&h[arr[i].x], 1u);
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    uint32_t r;
+    if (src.row(i, r)) atomicAdd(&h[r], 1u);
+  }
   __syncthreads();
   for (int r = threadIdx.x; r < nrows; r += blockDim.x)
     if (h[r]) atomicAdd(&row_cnt[r], h[r]);
@@ -126,13 +164,13 @@ static_assert(SCAN_THREADS * SCAN_LARGE == COUNT_SCAN_MAX, "one block holds ever
 constexpr int SC_THREADS = 512;
 constexpr int SC_PER = 16;
 constexpr int SC_CH = SC_THREADS * SC_PER;
-__global__ void __launch_bounds__(SC_THREADS) k_row_scatter(const Arrival* arr, const uint32_t* n_arr, uint32_t cap,
-                                                            const uint32_t* off, uint32_t* cursor, uint2* out,
+template <class Src>
+__global__ void __launch_bounds__(SC_THREADS) k_row_scatter(Src src, const uint32_t* off, uint32_t* cursor, uint2* out,
                                                             int nrows) {
   extern __shared__ uint32_t sm[];
   uint32_t* h = sm;           // per-row count in this chunk
   uint32_t* base = sm + nrows;
-  const uint32_t n = min(*n_arr, cap);
+  const uint32_t n = src.count();
   for (uint32_t c0 = blockIdx.x * SC_CH; c0 < n; c0 += gridDim.x * SC_CH) {
     for (int r = threadIdx.x; r < nrows; r += blockDim.x) h[r] = 0;
     __syncthreads();
@@ -142,11 +180,10 @@ __global__ void __launch_bounds__(SC_THREADS) k_row_scatter(const Arrival* arr, 
     for (int k = 0; k < SC_PER; ++k) {
       const uint32_t i = c0 + k * SC_THREADS + threadIdx.x;
       row[k] = 0xFFFFFFFFu;
-      if (i < n) {
-        const Arrival A = arr[i];
-        row[k] = A.x;
-        val[k] = make_uint2(A.y, A.z);
-        rank[k] = atomicAdd(&h[A.x], 1u);
+      uint32_t r;
+      if (i < n && src.get(i, r, val[k])) {
+        row[k] = r;
+        rank[k] = atomicAdd(&h[r], 1u);
       }
     }
     __syncthreads();
@@ -161,165 +198,171 @@ __global__ void __launch_bounds__(SC_THREADS) k_row_scatter(const Arrival* arr, 
 }
 
 // ------------------------------------------------------------------------------------------
-// 2. per row: sort by bin, segmented moment reduction, convolution
+// 2. per row: sort by bin, then, segment by segment of the record, segmented moment reduction and
+// convolution.  The moments of a whole 4096-sample row take 153 KB, one block per SM, whose
+// barriers and dependent passes nothing hid; a segment's take 78 KB, so two blocks of 512 threads
+// share an SM and overlap each other's phases.  A segment re-reduces its halo's arrivals (6 %).
+// The convolution's threads are 256 groups of 8 samples x 2 halves of the moments.  2048 rows of
+// 4096 samples, 7.9M arrivals: 459 -> 342 us (segments of 1024, three blocks: 345, and slower on
+// a hundred rows); 64 nearly empty rows 18.7 -> 16.7 us.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(ROW_THREADS) k_row_splat(SplatGeom g, const uint2* bucket, const uint32_t* off,
-                                                           uint2* scratch, const float* Gtab, float* rf) {
+__global__ void __launch_bounds__(ROW_THREADS, 2) k_row_splat(SplatGeom g, const uint2* bucket, const uint32_t* off,
+                                                              uint2* scratch, const float* Gtab, float* rf) {
   extern __shared__ float smf[];
   const int row = blockIdx.x;
   const int NB = g.nbins;         // bins -HALO .. ns + HALO - 1
-  const int MS = row_mom_stride(g.ns);
-  const int sh = row_mom_shift(g);  // bin x is stored at mom_slot(x + sh)
-  float* M = smf;                 // [K_MOM][MS], padded: one spare slot after every 8
-  uint32_t* hist = reinterpret_cast<uint32_t*>(M + K_MOM * MS);  // [NB + 1]
-  float* G = reinterpret_cast<float*>(hist + NB + 1);            // [K_MOM][MAX_TAPS], zero past ntaps
+  constexpr int MS = row_mom_stride(ROW_SEG);
+  const int sh = row_mom_shift(g);  // bin x of a segment is stored at mom_slot(x + sh)
+  float* M = smf;                 // [K_MOM][MS], padded: one spare slot after every 8; then the partial sums
+  float* G = M + K_MOM * MS;      // [K_MOM][MAX_TAPS], zero past ntaps
+  uint32_t* hist = reinterpret_cast<uint32_t*>(G + K_MOM * MAX_TAPS);  // [NB]
+  __shared__ uint32_t part[ROW_THREADS / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t a0 = off[row], a1 = off[row + 1];
-  for (int i = threadIdx.x; i < K_MOM * MS; i += blockDim.x) M[i] = 0.0f;
-  for (int i = threadIdx.x; i <= NB; i += blockDim.x) hist[i] = 0;
-  for (int i = threadIdx.x; i < K_MOM * MAX_TAPS; i += blockDim.x) {
+  float* out_row = rf + (size_t)row * g.ns;
+  if (a0 == a1) {  // nothing lands on this row
+    for (int n = tid; n < g.ns; n += ROW_THREADS) out_row[n] = 0.0f;
+    return;
+  }
+  for (int i = tid; i < NB; i += ROW_THREADS) hist[i] = 0;
+  for (int i = tid; i < K_MOM * MAX_TAPS; i += ROW_THREADS) {
     const int j = i / MAX_TAPS, d = i - j * MAX_TAPS;
     G[i] = d < g.ntaps ? Gtab[j * g.ntaps + d] : 0.0f;
   }
   __syncthreads();
   const uint32_t mask = (1u << TQ_FRAC) - 1u;
   // pass 1: histogram of bins
-  for (uint32_t i = a0 + threadIdx.x; i < a1; i += blockDim.x) {
+  for (uint32_t i = a0 + tid; i < a1; i += ROW_THREADS) {
     const int b = (int)(bucket[i].x >> TQ_FRAC) - TQ_OFFSET + HALO;
     if (b >= 0 && b < NB) atomicAdd(&hist[b], 1u);
   }
   __syncthreads();
-  // exclusive scan of hist (NB entries) in place: per-thread serial chunk + block scan
+  // exclusive scan of hist in place: a thread's own run of bins, then warps, then the block
   {
-    __shared__ uint32_t part[ROW_THREADS];
-    const int per = (NB + blockDim.x - 1) / blockDim.x;
-    const int lo = threadIdx.x * per, hi = min(NB, lo + per);
+    const int per = (NB + ROW_THREADS - 1) / ROW_THREADS;
+    const int lo = min(NB, tid * per), hi = min(NB, lo + per);
     uint32_t s = 0;
     for (int b = lo; b < hi; ++b) s += hist[b];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 1; o < (int)blockDim.x; o <<= 1) {
-      uint32_t v = threadIdx.x >= (unsigned)o ? part[threadIdx.x - o] : 0u;
-      __syncthreads();
-      part[threadIdx.x] += v;
-      __syncthreads();
+    uint32_t v = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, v, o);
+      if (lane >= o) v += u;
     }
-    uint32_t run = part[threadIdx.x] - s;
+    if (lane == 31) part[warp] = v;
+    __syncthreads();
+    uint32_t run = v - s + __reduce_add_sync(0xFFFFFFFFu, lane < warp ? part[lane & (ROW_THREADS / 32 - 1)] : 0u);
     for (int b = lo; b < hi; ++b) {
       const uint32_t c = hist[b];
       hist[b] = run;
       run += c;
     }
-    if (threadIdx.x == blockDim.x - 1) hist[NB] = part[threadIdx.x];
   }
   __syncthreads();
   // pass 2: scatter into bin order (scratch shares the row's index range)
-  for (uint32_t i = a0 + threadIdx.x; i < a1; i += blockDim.x) {
+  for (uint32_t i = a0 + tid; i < a1; i += ROW_THREADS) {
     const uint2 v = bucket[i];
     const int b = (int)(v.x >> TQ_FRAC) - TQ_OFFSET + HALO;
     if (b >= 0 && b < NB) scratch[a0 + atomicAdd(&hist[b], 1u)] = v;
   }
-  __syncthreads();
-  // after pass 2 hist[b] = end of bin b; total kept arrivals:
-  const uint32_t nk = hist[NB];
-  __syncthreads();
-  // pass 3: segmented warp reduction of the moments over the bin-sorted arrivals
-  const int lane = threadIdx.x & 31;
-  for (uint32_t base = (threadIdx.x & ~31u); base < nk; base += blockDim.x) {
-    const uint32_t i = base + lane;
-    int b = -1;
-    float m[K_MOM];
+  __syncthreads();  // from here hist[b] = end of bin b
+  for (int s0 = 0; s0 < g.ns; s0 += ROW_SEG) {  // samples s0 .. s0 + ROW_SEG - 1, bins s0 .. of the row's
+    const int b1 = min(NB, s0 + ROW_SEG + 2 * HALO);
+    const uint32_t r0 = s0 ? hist[s0 - 1] : 0u, r1 = hist[b1 - 1];
+    const int n_seg = min(ROW_SEG, g.ns - s0);
+    if (r0 == r1) {  // block-uniform
+      for (int n = tid; n < n_seg; n += ROW_THREADS) out_row[s0 + n] = 0.0f;
+      continue;
+    }
+    for (int i = tid; i < K_MOM * MS; i += ROW_THREADS) M[i] = 0.0f;
+    __syncthreads();
+    // segmented warp reduction of the moments over the bin-sorted arrivals
+    for (uint32_t base = r0 + (tid & ~31u); base < r1; base += ROW_THREADS) {
+      const uint32_t i = base + lane;
+      int b = -1;
+      float m[K_MOM];
 #pragma unroll
-    for (int j = 0; j < K_MOM; ++j) m[j] = 0.0f;
-    if (i < nk) {
-      const uint2 v = scratch[a0 + i];
-      b = (int)(v.x >> TQ_FRAC) - TQ_OFFSET + HALO;
-      const float delta = (float)(v.x & mask) * (1.0f / (float)(1u << TQ_FRAC)) - 0.5f;
-      float p = __uint_as_float(v.y);
-      m[0] = p;
+      for (int j = 0; j < K_MOM; ++j) m[j] = 0.0f;
+      if (i < r1) {
+        const uint2 v = scratch[a0 + i];
+        b = (int)(v.x >> TQ_FRAC) - TQ_OFFSET + HALO - s0;
+        const float delta = (float)(v.x & mask) * (1.0f / (float)(1u << TQ_FRAC)) - 0.5f;
+        float p = __uint_as_float(v.y);
+        m[0] = p;
 #pragma unroll
-      for (int j = 1; j < K_MOM; ++j) {
-        p = p * (-delta);  // the 1/j! of the Taylor term lives in the pulse table
-        m[j] = p;
+        for (int j = 1; j < K_MOM; ++j) {
+          p = p * (-delta);  // the 1/j! of the Taylor term lives in the pulse table
+          m[j] = p;
+        }
+      }
+      // inclusive segmented scan: lanes of one bin are contiguous (sorted)
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int bu = __shfl_up_sync(0xFFFFFFFFu, b, o);
+#pragma unroll
+        for (int j = 0; j < K_MOM; ++j) {
+          const float mu = __shfl_up_sync(0xFFFFFFFFu, m[j], o);
+          if (lane >= o && bu == b) m[j] += mu;
+        }
+      }
+      const int bn = __shfl_down_sync(0xFFFFFFFFu, b, 1);
+      const bool tail = (b >= 0) && (lane == 31 || bn != b);
+      if (tail) {
+#pragma unroll
+        for (int j = 0; j < K_MOM; ++j) atomicAdd(&M[j * MS + mom_slot(b + sh)], m[j]);
       }
     }
-    // inclusive segmented scan: lanes of one bin are contiguous (sorted)
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int bu = __shfl_up_sync(0xFFFFFFFFu, b, o);
-#pragma unroll
-      for (int j = 0; j < K_MOM; ++j) {
-        const float mu = __shfl_up_sync(0xFFFFFFFFu, m[j], o);
-        if (lane >= o && bu == b) m[j] += mu;
-      }
-    }
-    const int bn = __shfl_down_sync(0xFFFFFFFFu, b, 1);
-    const bool tail = (b >= 0) && (lane == 31 || bn != b);
-    if (tail) {
-#pragma unroll
-      for (int j = 0; j < K_MOM; ++j) atomicAdd(&M[j * MS + mom_slot(b + sh)], m[j]);
-    }
-  }
-  __syncthreads();
-  // convolution: each thread produces 8 consecutive samples n0 .. n0 + 7 of the row,
-  // out[n] = sum_j sum_d G_j[d] M_j[bin n - dlo - d].  Taps go in blocks of 8: the 15 moments a
-  // block touches are read once into registers (a sliding window) and feed 64 FMAs.  The
-  // shift sh puts every window start on a multiple of 8, so the padded slots of the window are
-  // fixed offsets and the lanes of a warp read addresses 9 apart: no bank conflicts.
-  const int n0 = 8 * threadIdx.x;
-  if (n0 < g.ns) {
+    __syncthreads();
+    // convolution: out[n] = sum_j sum_d G_j[d] M_j[bin n - dlo - d]; a thread produces 8 consecutive
+    // samples from two of the moments.  Taps go in blocks of 8: the 15 moments a block touches are
+    // read once into registers (a sliding window) and feed 64 FMAs.  The shift sh puts every
+    // window start on a multiple of 8, so the padded slots of the window are fixed offsets and
+    // the lanes of a warp read addresses 9 apart: no bank conflicts.
+    constexpr int GROUPS = ROW_SEG / 8, JG = ROW_THREADS / GROUPS;
+    const int n0 = 8 * (tid % GROUPS), jg = tid / GROUPS;
     float acc[8];
 #pragma unroll
     for (int r = 0; r < 8; ++r) acc[r] = 0.0f;
-    const int xs0 = n0 - g.dlo + HALO + sh - 7;  // window start for taps 0..7, a multiple of 8
-    const int ntp = (g.ntaps + 7) & ~7;
-    for (int j = 0; j < K_MOM; ++j) {
-      const float* Mj = M + j * MS;
-      const float* Gj = G + j * MAX_TAPS;
-      for (int d0 = 0; d0 < ntp; d0 += 8) {
-        const float* W = Mj + 9 * ((xs0 - d0) >> 3);
-        float w[15];
+    if (n0 < n_seg) {
+      const int xs0 = n0 - g.dlo + HALO + sh - 7;  // window start for taps 0..7, a multiple of 8
+      const int ntp = (g.ntaps + 7) & ~7;
+      for (int j = jg * (K_MOM / JG); j < (jg + 1) * (K_MOM / JG); ++j) {
+        const float* Mj = M + j * MS;
+        const float* Gj = G + j * MAX_TAPS;
+        for (int d0 = 0; d0 < ntp; d0 += 8) {
+          const float* W = Mj + 9 * ((xs0 - d0) >> 3);
+          float w[15];
 #pragma unroll
-        for (int k = 0; k < 15; ++k) w[k] = W[k + (k >= 8 ? 1 : 0)];
+          for (int k = 0; k < 15; ++k) w[k] = W[k + (k >= 8 ? 1 : 0)];
 #pragma unroll
-        for (int dd = 0; dd < 8; ++dd) {
-          const float gv = Gj[d0 + dd];
+          for (int dd = 0; dd < 8; ++dd) {
+            const float gv = Gj[d0 + dd];
 #pragma unroll
-          for (int r = 0; r < 8; ++r) acc[r] = fmaf(gv, w[r - dd + 7], acc[r]);
+            for (int r = 0; r < 8; ++r) acc[r] = fmaf(gv, w[r - dd + 7], acc[r]);
+          }
         }
       }
     }
-    float* out = rf + (size_t)row * g.ns + n0;
-    if (n0 + 8 <= g.ns) {
-      reinterpret_cast<float4*>(out)[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-      reinterpret_cast<float4*>(out)[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
-    } else {
+    __syncthreads();
+    float* P = M;  // [JG][GROUPS * 9]: the moment groups' sums, one spare slot after every 8
 #pragma unroll
-      for (int r = 0; r < 8; ++r)
-        if (n0 + r < g.ns) out[r] = acc[r];
+    for (int r = 0; r < 8; ++r) P[jg * (GROUPS * 9) + (n0 / 8) * 9 + r] = acc[r];
+    __syncthreads();
+    for (int n = tid; n < n_seg; n += ROW_THREADS) {
+      float v = 0.0f;
+#pragma unroll
+      for (int k = 0; k < JG; ++k) v += P[k * (GROUPS * 9) + mom_slot(n)];
+      out_row[s0 + n] = v;
     }
-  }
-}
-
-// standalone arrival list -> packed arrivals
-__global__ void k_pack_arrivals(const int32_t* tx, const int32_t* e, const float* tau, const float* a, long long n,
-                                int ne, float fs, Arrival* out, uint32_t* n_out) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const uint32_t tq = time_to_tq(tau[i], 0.0f, fs);
-    if (tq == 0xFFFFFFFFu) continue;
-    cg::coalesced_group grp = cg::coalesced_threads();
-    uint32_t s = 0;
-    if (grp.thread_rank() == 0) s = atomicAdd(n_out, (uint32_t)grp.size());
-    s = grp.shfl(s, 0) + grp.thread_rank();
-    out[s] = make_uint4((uint32_t)(tx[i] * ne + e[i]), tq, __float_as_uint(a[i]), (uint32_t)i);
+    __syncthreads();
   }
 }
 
 // ------------------------------------------------------------------------------------------
 size_t row_splat_smem(const SplatGeom& g) {
-  return sizeof(float) * (size_t)K_MOM * row_mom_stride(g.ns) + sizeof(uint32_t) * (g.nbins + 1) +
+  return sizeof(float) * (size_t)K_MOM * row_mom_stride(ROW_SEG) + sizeof(uint32_t) * g.nbins +
          sizeof(float) * (size_t)K_MOM * MAX_TAPS;
 }
-int row_splat_threads(const SplatGeom& g) { return ((g.ns + 7) / 8 + 31) / 32 * 32; }
 
 void launch_pulse_table(const SplatGeom& g, float* G, cudaStream_t st) { k_pulse_table<<<1, 128, 0, st>>>(g, G); }
 
@@ -330,34 +373,40 @@ void launch_count_scan(const uint32_t* cnt, uint32_t* off, uint32_t* cursor, int
     k_row_scan<SCAN_LARGE><<<1, SCAN_THREADS, 0, st>>>(cnt, off, cursor, n);
 }
 
-void launch_splat_sort(const SplatGeom& g, const Arrival* arr, const uint32_t* n_arr, uint32_t cap, SplatWork w,
-                       int grid, cudaStream_t st) {
+template <class Src>
+static void splat_sort(const SplatGeom& g, const Src& src, SplatWork w, int grid, cudaStream_t st) {
   const int nrows = g.nrows;
   cudaMemsetAsync(w.row_cnt, 0, sizeof(uint32_t) * nrows, st);
-  k_row_hist<<<grid, 256, sizeof(uint32_t) * nrows, st>>>(arr, n_arr, cap, w.row_cnt, nrows);
+  k_row_hist<<<grid, 256, sizeof(uint32_t) * nrows, st>>>(src, w.row_cnt, nrows);
   launch_count_scan(w.row_cnt, w.row_off, w.row_cursor, nrows, st);
-  k_row_scatter<<<grid, SC_THREADS, 2 * sizeof(uint32_t) * nrows, st>>>(arr, n_arr, cap, w.row_off, w.row_cursor,
-                                                                         w.bucket, nrows);
+  k_row_scatter<<<grid, SC_THREADS, 2 * sizeof(uint32_t) * nrows, st>>>(src, w.row_off, w.row_cursor, w.bucket, nrows);
+}
+void launch_splat_sort(const SplatGeom& g, const Arrival* arr, const uint32_t* n_arr, uint32_t cap, SplatWork w,
+                       int grid, cudaStream_t st) {
+  splat_sort(g, PackedArrivals{arr, n_arr, cap}, w, grid, st);
+}
+void launch_splat_sort_list(const SplatGeom& g, const int32_t* tx, const int32_t* e, const float* tau, const float* a,
+                            uint32_t n, int ne, float fs, SplatWork w, int grid, cudaStream_t st) {
+  splat_sort(g, ListedArrivals{tx, e, tau, a, n, ne, fs}, w, grid, st);
 }
 void launch_splat_rows(const SplatGeom& g, SplatWork w, const float* G, float* rf, cudaStream_t st) {
-  k_row_splat<<<g.nrows, row_splat_threads(g), row_splat_smem(g), st>>>(g, w.bucket, w.row_off, w.scratch, G, rf);
-}
-
-void launch_pack_arrivals(const int32_t* tx, const int32_t* e, const float* tau, const float* a, long long n, int ne,
-                          float fs, Arrival* out, uint32_t* n_out, int grid, cudaStream_t st) {
-  k_pack_arrivals<<<grid, 256, 0, st>>>(tx, e, tau, a, n, ne, fs, out, n_out);
+  k_row_splat<<<g.nrows, ROW_THREADS, row_splat_smem(g), st>>>(g, w.bucket, w.row_off, w.scratch, G, rf);
 }
 
 cudaError_t splat_set_attrs(const SplatGeom& g) {
   return cudaFuncSetAttribute(k_row_splat, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_splat_smem(g));
 }
 cudaError_t row_scatter_set_attrs(int nrows) {
-  return cudaFuncSetAttribute(k_row_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(2 * sizeof(uint32_t) * nrows));
+  const int sm = (int)(2 * sizeof(uint32_t) * nrows);
+  const cudaError_t e = cudaFuncSetAttribute(k_row_scatter<PackedArrivals>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_row_scatter<ListedArrivals>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
 }
 cudaError_t row_hist_set_attrs(int nrows) {
-  return cudaFuncSetAttribute(k_row_hist, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(sizeof(uint32_t) * nrows));
+  const int sm = (int)(sizeof(uint32_t) * nrows);
+  const cudaError_t e = cudaFuncSetAttribute(k_row_hist<PackedArrivals>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_row_hist<ListedArrivals>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
 }
 
 }  // namespace usrt
