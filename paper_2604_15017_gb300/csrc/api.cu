@@ -845,7 +845,7 @@ int us_scene_upload(us_ctx* ctx, const us_scene_desc* d, uint64_t* scene_id) {
       (s = up(o.tri_e2, &sc.dev.tri_e2)) || (s = up(o.scat, &sc.dev.scat)) ||
       (s = up(o.nodes_t, &sc.dev.nodes_t)) || (s = up(o.prims_t, &sc.dev.prims_t)) ||
       (s = up(o.nodes4, &sc.dev.nodes4)) ||
-      (s = up(o.cell_rec, &sc.dev.cell_rec))) {
+      (s = up_bytes(o.cell_rec.data(), o.cell_rec.size() * sizeof(float), reinterpret_cast<const void**>(&sc.dev.cell_rec)))) {
     for (void* p : sc.allocs) cudaFree(p);
     ctx->used -= sc.bytes;
     return s;

@@ -442,7 +442,7 @@ static void build_scatter_grid(const HostSceneIn& in, HostSceneOut& out) {
     if (most > 255 || acc >= (1u << 24)) continue;
     // chain records of crowded cells follow the cells' own; entries fill a chain in order
     out.cell_rec.assign(8 * n_recs, REC_EMPTY);
-    for (size_t r = 0; r < n_recs; ++r) out.cell_rec[8 * r + 3] = out.cell_rec[8 * r + 7] = 0.0f;
+    for (size_t r = 0; r < n_recs; ++r) out.cell_rec[8 * r + 6] = out.cell_rec[8 * r + 7] = 0.0f;
     std::vector<uint32_t> tail(n_cells), filled(n_cells, 0);
     for (size_t c = 0; c < n_cells; ++c) tail[c] = (uint32_t)c;
     uint32_t n_chain = 0;  // at most acc / 2 < 2^23
@@ -451,19 +451,19 @@ static void build_scatter_grid(const HostSceneIn& in, HostSceneOut& out) {
         if (filled[c] == 2) {
           float* r = &out.cell_rec[8 * (size_t)tail[c]];
           uint32_t w0, w1;
-          std::memcpy(&w0, &r[3], 4);
+          std::memcpy(&w0, &r[6], 4);
           std::memcpy(&w1, &r[7], 4);
           ++n_chain;
-          r[3] = bits_f(w0 | (n_chain >> 12) << 20);
+          r[6] = bits_f(w0 | (n_chain >> 12) << 20);
           r[7] = bits_f(w1 | (n_chain & 0xFFFu) << 20);
           tail[c] = (uint32_t)n_cells + n_chain - 1;
           filled[c] = 0;
         }
-        float* e = &out.cell_rec[8 * (size_t)tail[c] + 4 * filled[c]++];
-        e[0] = in.scat_pos[3 * (size_t)j];
-        e[1] = in.scat_pos[3 * (size_t)j + 1];
-        e[2] = in.scat_pos[3 * (size_t)j + 2];
-        e[3] = bits_f((uint32_t)j);
+        float* e = &out.cell_rec[8 * (size_t)tail[c] + filled[c]++];
+        e[0] = -in.scat_pos[3 * (size_t)j];
+        e[2] = -in.scat_pos[3 * (size_t)j + 1];
+        e[4] = -in.scat_pos[3 * (size_t)j + 2];
+        e[6] = bits_f((uint32_t)j);
       });
     return;
   }

@@ -24,10 +24,11 @@ struct HostSceneOut {
   std::vector<float> nodes4;       // 32 floats per node
   // uniform grid over the scatterer spheres: cell (x, y, z) covers glo + h [x, x+1) x [y, y+1) x
   // [z, z+1) and lists every sphere whose (slightly inflated) bounding box overlaps it, in
-  // records of two 16-byte entries (centre, sphere id | part of `next` << 20).  Record
-  // (z * gn[1] + y) * gn[0] + x is the cell's first; `next`, 24 bits (the high 12 in the first
-  // entry, the low 12 in the second), names the record that follows in a crowded cell, record
-  // (number of cells) + next - 1, or is 0.  An empty entry's centre is NaN.
+  // records of two entries a, b: (-xa, -xb, -ya, -yb, -za, -zb, wa, wb), the negated centres side
+  // by side for packed arithmetic, w the sphere id | part of `next` << 20.  Record
+  // (z * gn[1] + y) * gn[0] + x is the cell's first; `next`, 24 bits (the high 12 in wa, the low 12
+  // in wb), names the record that follows in a crowded cell, record (number of cells) + next - 1,
+  // or is 0.  An empty entry's centre is NaN.
   float glo[3] = {0, 0, 0}, gh = 1.0f;
   int gn[3] = {0, 0, 0};
   std::vector<float> cell_rec;  // 8 floats per record

@@ -57,18 +57,52 @@ __device__ __forceinline__ float tri_test(float3 o, float3 w, float3 v0, float3 
   return t > T_MIN ? t : -1.0f;
 }
 
-// point scatterer: event at the closest approach t = (p - o).w when within r_s of the centre
-// The roundings are spelled out: whether a ray passes within r_s is a decision, and left to the
-// compiler's choice of fused products it changed with the code around it (6 of 16 million paths)
-__device__ __forceinline__ float dot3_rn(float3 a, float3 b) {
-  return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));
+// two FP32 values in one 64-bit register and the packed instructions on them (one issue slot for two
+// rounded operations)
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
 }
-__device__ __forceinline__ float scat_test(float3 o, float3 w, float3 p, float rs2) {
-  const float3 d = p - o;
-  const float t = dot3_rn(d, w);
-  if (!(t > T_MIN)) return -1.0f;
-  const float3 q = f3(__fmaf_rn(w.x, t, -d.x), __fmaf_rn(w.y, t, -d.y), __fmaf_rn(w.z, t, -d.z));
-  return dot3_rn(q, q) <= rs2 ? t : -1.0f;
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// Point scatterers, two at a time: with d = p - o, the closest approach t = d.w, and the squared
+// distance |w t - d|^2 there (an event when that is within r_s and t > T_MIN).  The centres are
+// given negated, so that -d is one addition; both factors' signs drop out exactly.  The roundings
+// are spelled out: whether a ray passes within r_s is a decision, and left to the compiler's
+// choice of fused products it changed with the code around it (6 of 16 million paths).
+struct Ray2 {
+  f32x2 ox, oy, oz, wx, wy, wz;  // origin and direction, each twice
+};
+__device__ __forceinline__ Ray2 ray2(float3 o, float3 w) {
+  return Ray2{pack2(o.x, o.x), pack2(o.y, o.y), pack2(o.z, o.z), pack2(w.x, w.x), pack2(w.y, w.y), pack2(w.z, w.z)};
+}
+__device__ __forceinline__ void scat_test2(const Ray2& r, f32x2 npx, f32x2 npy, f32x2 npz, float2& t, float2& dist2) {
+  const f32x2 x = add2(npx, r.ox), y = add2(npy, r.oy), z = add2(npz, r.oz);  // -d
+  const f32x2 tt = fma2(z, r.wz, fma2(x, r.wx, mul2(y, r.wy))) ^ 0x8000000080000000ull;
+  const f32x2 qx = fma2(r.wx, tt, x), qy = fma2(r.wy, tt, y), qz = fma2(r.wz, tt, z);
+  t = unpack2(tt);
+  dist2 = unpack2(fma2(qz, qz, fma2(qx, qx, mul2(qy, qy))));
 }
 
 __device__ __forceinline__ bool hit_better(float t, uint32_t c, float tb, uint32_t cb) {

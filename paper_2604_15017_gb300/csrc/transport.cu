@@ -191,16 +191,20 @@ __global__ void __launch_bounds__(TRAV_THREADS, 8) k_traverse(TransportArgs A) {
 // kernel lasts as long as its longest chain of iterations, so the rays are spread over all
 // resident warps, a few lanes each (warp_lanes).
 //
-// Bound by the latency of that chain: one L2 record read and ~70 instructions per iteration.  Per
-// inclusion frame (38M rays, 1.1e9 cells) closest hits took 19.3 ms when a crowded cell's entries
-// were looked up and tested one by one (its lanes' two further dependent reads held up the whole
-// warp in most iterations) and a step kept three cell coordinates; 16.6 ms so.  Five rounds of
-// 1e5 .. 1e4 rays: 1424 -> 790 us.
+// Bound by instruction issue and the latency of that chain about equally: one L2 record read and
+// ~55 instructions per iteration, the two spheres tested side by side in packed FP32
+// (scat_test2), the rare one that is passed within r_s sorted out behind a branch.  72 registers, 7
+// blocks per SM (64: spills, frame +1.4 ms; 80: +0.5 ms); two records per look at the idle lanes:
+// +1.2 ms.  Per inclusion frame (38M rays, 1.1e9 cells) closest hits took 19.3 ms when a crowded
+// cell's entries were looked up and tested one by one (its lanes' two further dependent reads
+// held up the whole warp in most iterations) and a step kept three cell coordinates, 16.6 with the
+// chained records, 15.3 with coarser cells, 14.1 with the packed tests.  Five rounds of 1e5 .. 1e4
+// rays: 1424 us, 790, 680, with the joint launch 408, now 375.
 // ------------------------------------------------------------------------------------------
-// 32-ray claims and a refill at 4 idle lanes, measured against 64 and 128 rays, 8, 12 and 16 lanes
-// (medium render 927 us of closest hits against 977 with 64-ray claims; the frame is indifferent)
+// 32-ray claims and a refill at 8 idle lanes, measured against 64 and 128 rays, 4, 6, 12 and 16 lanes
+// (inclusion frame 23.0 ms with 4 lanes, 22.7 with 6, 22.5 with 8)
 constexpr int MARCH_CHUNK = 32;
-constexpr int MARCH_REFILL_MIN = 4;
+constexpr int MARCH_REFILL_MIN = 8;
 
 // block `block` of `blocks` resident ones.  JOINT: rays before `unbounded`, whose surface hit is not
 // known yet, are searched to the end of the grid, and every ray's scat is written (t = 3e38:
@@ -223,27 +227,18 @@ __device__ __forceinline__ void march_rays(const TransportArgs& A, uint32_t bloc
   const int nx = S.gnx, ny = S.gny, nz = S.gnz;
   // lane state
   uint32_t ray = 0xFFFFFFFFu;  // queue slot of the current ray; none when 0xFFFFFFFF
-  float3 o = f3(0.0f, 0.0f, 0.0f), w = o;
-  // per axis: the next face (tn = fma(k, dt, t_0)), its step number k, dt, t_0, the cell stride
-  float tnx = 0.0f, tny = 0.0f, tnz = 0.0f, kx = 0.0f, ky = 0.0f, kz = 0.0f;
+  Ray2 r2 = ray2(f3(0.0f, 0.0f, 0.0f), f3(0.0f, 0.0f, 0.0f));
+  // per axis: the step number k of the next face (at t_0 + k dt), dt, t_0, the cell stride
+  float kx = 0.0f, ky = 0.0f, kz = 0.0f;
   float dtx = 0.0f, dty = 0.0f, dtz = 0.0f, fx = 0.0f, fy = 0.0f, fz = 0.0f;
   int sx = 0, sy = 0, sz = 0, cell = 0;
   float tbest = 0.0f, tend = 0.0f;
   uint32_t prev = 0u, cbest = 0u;
   constexpr uint32_t NO_SCAT = 0u;  // before every code: a scatterer at the bound itself is none
-  float4 slot_a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), slot_b = slot_a;  // the record to test next
+  ulonglong2 rec_a = make_ulonglong2(0ull, 0ull), rec_b = rec_a;  // the record to test next
   auto fetch = [&](int rec) {
-    slot_a = __ldg(&S.cell_rec[2 * (size_t)rec]);
-    slot_b = __ldg(&S.cell_rec[2 * (size_t)rec + 1]);
-  };
-  auto test = [&](float4 sp) {
-    const uint32_t id = __float_as_uint(sp.w) & 0xFFFFFu;
-    const float t = scat_test(o, w, xyz(sp), S.rs2);
-    const uint32_t code = prim_code(CLS_SCAT, id);
-    if (t > 0.0f && code != prev && hit_better(t, code, tbest, cbest)) {
-      tbest = t;
-      cbest = code;
-    }
+    rec_a = __ldg(&S.cell_rec[2 * (size_t)rec]);
+    rec_b = __ldg(&S.cell_rec[2 * (size_t)rec + 1]);
   };
   // the first chunk of every warp is its own; the counter hands out the ones after those
   uint32_t pool = min(n, (block + blocks * (threadIdx.x >> 5)) * chunk);  // warp-uniform
@@ -274,14 +269,14 @@ __device__ __forceinline__ void march_rays(const TransportArgs& A, uint32_t bloc
         ray = pool + rank;
         const float4 pa = A.qin.pa[ray];
         const float4 wt = A.qin.wt[ray];
+        const float3 o = xyz(pa), w = xyz(wt);
+        r2 = ray2(o, w);
         if (JOINT && !A.sort) {
           tbest = A.qin.surf[ray].x;  // carried, or none
           if (tbest < 0.0f) tbest = 3.0e38f;
         } else {
           tbest = JOINT && ray < unbounded ? 3.0e38f : A.hits[ray].x;
         }
-        o = xyz(pa);
-        w = xyz(wt);
         prev = A.qin.meta[ray].y;
         cbest = NO_SCAT;
         const float ix = safe_inv(w.x), iy = safe_inv(w.y), iz = safe_inv(w.z);
@@ -307,9 +302,9 @@ __device__ __forceinline__ void march_rays(const TransportArgs& A, uint32_t bloc
           dtx = fminf(h * fabsf(ix), 1e30f);
           dty = fminf(h * fabsf(iy), 1e30f);
           dtz = fminf(h * fabsf(iz), 1e30f);
-          tnx = fx = fmaxf((fmaf((float)(cx + (ux ? 1 : 0)), h, lo.x) - o.x) * ix, -3e38f);
-          tny = fy = fmaxf((fmaf((float)(cy + (uy ? 1 : 0)), h, lo.y) - o.y) * iy, -3e38f);
-          tnz = fz = fmaxf((fmaf((float)(cz + (uz ? 1 : 0)), h, lo.z) - o.z) * iz, -3e38f);
+          fx = fmaxf((fmaf((float)(cx + (ux ? 1 : 0)), h, lo.x) - o.x) * ix, -3e38f);
+          fy = fmaxf((fmaf((float)(cy + (uy ? 1 : 0)), h, lo.y) - o.y) * iy, -3e38f);
+          fz = fmaxf((fmaf((float)(cz + (uz ? 1 : 0)), h, lo.z) - o.z) * iz, -3e38f);
           // past the last face along an axis the ray is outside: no cell is entered at or after
           // tend, and t_0 + k dt < tend only for faces before the last
           tend = fminf(fminf(fmaf((float)(ux ? nx - 1 - cx : cx), dtx, fx), fmaf((float)(uy ? ny - 1 - cy : cy), dty, fy)),
@@ -327,30 +322,32 @@ __device__ __forceinline__ void march_rays(const TransportArgs& A, uint32_t bloc
     }
     if (__all_sync(0xFFFFFFFFu, ray == 0xFFFFFFFFu)) break;  // pool exhausted, every lane idle
     if (ray == 0xFFFFFFFFu) continue;
-    test(slot_a);
-    test(slot_b);
+    float2 t2, d2;
+    scat_test2(r2, rec_a.x, rec_a.y, rec_b.x, t2, d2);
+    const uint32_t ia = (uint32_t)rec_b.y, ib = (uint32_t)(rec_b.y >> 32);
+    if (d2.x <= S.rs2 || d2.y <= S.rs2) {  // one record in twenty
+      const uint32_t ca = prim_code(CLS_SCAT, ia & 0xFFFFFu), cb = prim_code(CLS_SCAT, ib & 0xFFFFFu);
+      if (d2.x <= S.rs2 && t2.x > T_MIN && ca != prev && hit_better(t2.x, ca, tbest, cbest)) {
+        tbest = t2.x;
+        cbest = ca;
+      }
+      if (d2.y <= S.rs2 && t2.y > T_MIN && cb != prev && hit_better(t2.y, cb, tbest, cbest)) {
+        tbest = t2.y;
+        cbest = cb;
+      }
+    }
     // the record after this one: the next of a crowded cell's chain, or the next cell's
-    int rec = (int)((__float_as_uint(slot_a.w) >> 20 << 12) | (__float_as_uint(slot_b.w) >> 20));
+    int rec = (int)((ia >> 20 << 12) | (ib >> 20));
     if (rec != 0) {
       rec += nx * ny * nz - 1;
     } else {
-      float t;
-      if (tnx <= tny && tnx <= tnz) {
-        t = tnx;
-        cell += sx;
-        kx += 1.0f;
-        tnx = fmaf(kx, dtx, fx);
-      } else if (tny <= tnz) {
-        t = tny;
-        cell += sy;
-        ky += 1.0f;
-        tny = fmaf(ky, dty, fy);
-      } else {
-        t = tnz;
-        cell += sz;
-        kz += 1.0f;
-        tnz = fmaf(kz, dtz, fz);
-      }
+      const float tnx = fmaf(kx, dtx, fx), tny = fmaf(ky, dty, fy), tnz = fmaf(kz, dtz, fz);
+      const float t = fminf(tnx, fminf(tny, tnz));
+      const bool px = tnx <= fminf(tny, tnz), py = !px && tny <= tnz;
+      cell += px ? sx : (py ? sy : sz);
+      if (px) kx += 1.0f;
+      if (py) ky += 1.0f;
+      if (!px && !py) kz += 1.0f;
       if (!(t <= tbest && t < tend)) {  // no cell left to enter below tbest: done
         if (JOINT) {
           A.scat[ray] = make_float2(cbest != NO_SCAT ? tbest : 3.0e38f, __uint_as_float(cbest));
@@ -367,7 +364,7 @@ __device__ __forceinline__ void march_rays(const TransportArgs& A, uint32_t bloc
   }
 }
 
-__global__ void __launch_bounds__(MARCH_THREADS, 8) k_march(TransportArgs A) {
+__global__ void __launch_bounds__(MARCH_THREADS, 7) k_march(TransportArgs A) {
   if (A.cnt->live[A.k] > 0u) march_rays<false>(A, blockIdx.x, gridDim.x, 0u);
 }
 
@@ -375,7 +372,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, 8) k_march(TransportArgs A) {
 // blocks walk the BVH, the second half march the grid, without the surface bound for the rays
 // whose surface hit is not known yet.  Such a round lasts as long as the longest chain of
 // either search, so what the missing bound adds does not show, and the two chains overlap.
-__global__ void __launch_bounds__(TRAV_THREADS, 8) k_closest(TransportArgs A) {
+__global__ void __launch_bounds__(TRAV_THREADS, 7) k_closest(TransportArgs A) {
   const uint32_t half = gridDim.x / 2;
   if (blockIdx.x < half)
     traverse_rays(A, blockIdx.x, half, 1u);

@@ -89,7 +89,7 @@ struct SceneDev {
                              // n2=(c0 z, c1 z) n3=int4(child0, child1, count0, count1)
   const float4* prims_t;     // triangles in leaf order: (v0, code) (e1, -) (e2, -)
   const float4* nodes4;      // the triangle tree as a 4-wide BVH (8 float4 per node, same leaves)
-  const float4* cell_rec;      // scatterer grid: records of two entries (centre, id | next bits << 20),
+  const ulonglong2* cell_rec;  // scatterer grid: records of two entries, two words of 16 bytes each,
                                // cell (z * gny + y) * gnx + x first, then the crowded cells' chains
   float3 glo;                  // grid origin and cell edge
   float gh;
