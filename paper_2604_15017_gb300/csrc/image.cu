@@ -677,25 +677,49 @@ __global__ void __launch_bounds__(DJ_THREADS) k_das_adj_tile(Acq q, Img im, int 
 }
 
 // ------------------------------------------------------------------------------------------
-// shared-memory radix-2 FFT of one line (N = n_depth, power of two)
+// shared-memory FFT of one line (N = n_depth, power of two): radix-2 butterflies, R consecutive
+// stages at a time in the registers of one thread (the same butterflies with the same roundings
+// as one stage at a time), so that a line of 1024 has 5 barriers per transform instead of 10.
+// A line's transforms are bound by those barriers' latencies.
 // ------------------------------------------------------------------------------------------
-__device__ void fft_smem(float2* z, const float2* tw, int N, int logN, bool inverse) {
-  for (int len = 2, s = 1; len <= N; len <<= 1, ++s) {
-    const int half = len >> 1;
-    const int step = N >> s;
-    for (int b = threadIdx.x; b < (N >> 1); b += blockDim.x) {
-      const int grp = b >> (s - 1);
-      const int kk = b & (half - 1);
-      const int i = grp * len + kk, j = i + half;
-      float2 w = tw[kk * step];
-      if (inverse) w.y = -w.y;
-      const float2 xj = z[j], xi = z[i];
-      const float2 t = make_float2(w.x * xj.x - w.y * xj.y, w.x * xj.y + w.y * xj.x);
-      z[j] = make_float2(xi.x - t.x, xi.y - t.y);
-      z[i] = make_float2(xi.x + t.x, xi.y + t.y);
+// slot of z[i]: one spare after every 16, so that strided groups spread over the banks
+__host__ __device__ constexpr int fft_slot(int i) { return i + (i >> 4); }
+__host__ __device__ constexpr size_t fft_line_bytes(int N) { return sizeof(float2) * (size_t)(fft_slot(N) + 1); }
+
+template <int R, bool INVERSE>
+__device__ __forceinline__ void fft_pass(float2* z, const float2* tw, int N, int s) {  // stages s .. s + R - 1 (from 1)
+  constexpr int E = 1 << R;
+  const int half = 1 << (s - 1);
+  for (int g = threadIdx.x; g < (N >> R); g += blockDim.x) {
+    const int kk = g & (half - 1), base = ((g >> (s - 1)) << (s - 1 + R)) + kk;
+    float2 v[E];
+#pragma unroll
+    for (int j = 0; j < E; ++j) v[j] = z[fft_slot(base + j * half)];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+#pragma unroll
+      for (int j = 0; j < E; ++j) {
+        if (j & (1 << r)) continue;
+        float2 w = tw[(kk + (j & ((1 << r) - 1)) * half) * (N >> (s + r))];
+        if (INVERSE) w.y = -w.y;
+        const float2 xi = v[j], xj = v[j + (1 << r)];
+        const float2 t = make_float2(w.x * xj.x - w.y * xj.y, w.x * xj.y + w.y * xj.x);
+        v[j + (1 << r)] = make_float2(xi.x - t.x, xi.y - t.y);
+        v[j] = make_float2(xi.x + t.x, xi.y + t.y);
+      }
     }
-    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < E; ++j) z[fft_slot(base + j * half)] = v[j];
   }
+  __syncthreads();
+}
+template <bool INVERSE>
+__device__ void fft_smem(float2* z, const float2* tw, int N, int logN) {
+  int s = 1;
+  if (N >= 2048)  // as many groups of 8 as threads
+    for (; s + 2 <= logN; s += 3) fft_pass<3, INVERSE>(z, tw, N, s);
+  for (; s + 1 <= logN; s += 2) fft_pass<2, INVERSE>(z, tw, N, s);
+  if (s <= logN) fft_pass<1, INVERSE>(z, tw, N, s);
 }
 
 __device__ void twiddles(float2* tw, int N) {
@@ -705,27 +729,32 @@ __device__ void twiddles(float2* tw, int N) {
     tw[kk] = make_float2(c, s);
   }
 }
+__device__ __forceinline__ int bit_rev(int i, int logN) { return (int)(__brev((unsigned)i) >> (32 - logN)); }
 
 // analytic signal of a real line (already bit-reversed into z): X = FFT(x); X *= h; IFFT / N
 __device__ void analytic_smem(float2* z, const float2* tw, int N, int logN) {
-  fft_smem(z, tw, N, logN, false);
-  for (int kk = threadIdx.x; kk < N; kk += blockDim.x) {
-    const float h = (kk == 0 || 2 * kk == N) ? 1.0f : (2 * kk < N ? 2.0f : 0.0f);
-    const float sc = h / (float)N;
-    z[kk] = make_float2(z[kk].x * sc, z[kk].y * sc);
-  }
-  __syncthreads();
-  // bit-reverse in place for the inverse transform
+  fft_smem<false>(z, tw, N, logN);
+  // scale and bit-reverse in place for the inverse transform, a pair of slots per thread
+  auto scale = [&](int kk) { return ((kk == 0 || 2 * kk == N) ? 1.0f : (2 * kk < N ? 2.0f : 0.0f)) / (float)N; };
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    const int j = (int)(__brev((unsigned)i) >> (32 - logN));
-    if (i < j) {
-      const float2 t = z[i];
-      z[i] = z[j];
-      z[j] = t;
-    }
+    const int j = bit_rev(i, logN);
+    if (i > j) continue;
+    const float si = scale(i), sj = scale(j);
+    const float2 a = z[fft_slot(i)], b = z[fft_slot(j)];
+    z[fft_slot(i)] = make_float2(b.x * sj, b.y * sj);
+    z[fft_slot(j)] = make_float2(a.x * si, a.y * si);
   }
   __syncthreads();
-  fft_smem(z, tw, N, logN, true);
+  fft_smem<true>(z, tw, N, logN);
+}
+// largest key of the block into *best (every thread calls; one shared atomic per warp)
+__device__ __forceinline__ void block_max_key(unsigned long long key, unsigned long long* best) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long k = __shfl_xor_sync(0xFFFFFFFFu, key, o);
+    key = k > key ? k : key;
+  }
+  if ((threadIdx.x & 31) == 0 && key) atomicMax(best, key);
 }
 
 // envelope of each line: E = |x + i H x|; per-image maximum (value, first index) into a
@@ -735,27 +764,28 @@ __global__ void k_envelope(Img im, const float* __restrict__ irf, float* env, un
   const int N = im.nd;
   const int logN = 31 - __clz(N);
   float2* z = sz;
-  float2* tw = sz + N;
+  float2* tw = sz + fft_slot(N) + 1;
   twiddles(tw, N);
   __shared__ unsigned long long best;
   if (threadIdx.x == 0) best = 0ull;
+  unsigned long long own = 0ull;
   for (int l = blockIdx.x; l < im.nl; l += gridDim.x) {
     const float* x = irf + (size_t)l * N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const int j = (int)(__brev((unsigned)i) >> (32 - logN));
-      z[j] = make_float2(__ldg(&x[i]), 0.0f);
-    }
+    for (int i = threadIdx.x; i < N; i += blockDim.x) z[fft_slot(bit_rev(i, logN))] = make_float2(__ldg(&x[i]), 0.0f);
     __syncthreads();
     analytic_smem(z, tw, N, logN);
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const float e = sqrtf(z[i].x * z[i].x + z[i].y * z[i].y);
+      const float2 v = z[fft_slot(i)];
+      const float e = sqrtf(v.x * v.x + v.y * v.y);
       env[(size_t)l * N + i] = e;
       const unsigned long long key =
           ((unsigned long long)__float_as_uint(e) << 32) | (0xFFFFFFFFu - (uint32_t)(l * N + i));
-      atomicMax(&best, key);
+      own = key > own ? key : own;
     }
     __syncthreads();
   }
+  block_max_key(own, &best);
+  __syncthreads();
   if (threadIdx.x == 0) atomicMax(emax_key, best);
 }
 
@@ -782,27 +812,30 @@ __global__ void k_envlog_fused(Img im, const float* __restrict__ irf, unsigned l
   const int N = im.nd;
   const int logN = 31 - __clz(N);
   float2* z = sz;
-  float2* tw = sz + N;
+  float2* tw = sz + fft_slot(N) + 1;
   float* ev = reinterpret_cast<float*>(tw + N / 2);  // envelopes of this block's lines
   twiddles(tw, N);
   __shared__ unsigned long long best;
   if (threadIdx.x == 0) best = 0ull;
+  unsigned long long own = 0ull;
   int j = 0;
   for (int l = blockIdx.x; l < im.nl; l += gridDim.x, ++j) {
     const float* x = irf + (size_t)l * N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const int r = (int)(__brev((unsigned)i) >> (32 - logN));
-      z[r] = make_float2(__ldg(&x[i]), 0.0f);
-    }
+    for (int i = threadIdx.x; i < N; i += blockDim.x) z[fft_slot(bit_rev(i, logN))] = make_float2(__ldg(&x[i]), 0.0f);
     __syncthreads();
     analytic_smem(z, tw, N, logN);
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const float e = sqrtf(z[i].x * z[i].x + z[i].y * z[i].y);
+      const float2 v = z[fft_slot(i)];
+      const float e = sqrtf(v.x * v.x + v.y * v.y);
       ev[j * N + i] = e;
-      atomicMax(&best, ((unsigned long long)__float_as_uint(e) << 32) | (0xFFFFFFFFu - (uint32_t)(l * N + i)));
+      const unsigned long long key =
+          ((unsigned long long)__float_as_uint(e) << 32) | (0xFFFFFFFFu - (uint32_t)(l * N + i));
+      own = key > own ? key : own;
     }
     __syncthreads();
   }
+  block_max_key(own, &best);
+  __syncthreads();
   bool ok = true;
   if (threadIdx.x == 0) {
     atomicMax(&keyw[0], best);
@@ -908,8 +941,8 @@ __global__ void k_envlog_vjp(Img im, const float* __restrict__ irf, const float*
   const int N = im.nd;
   const int logN = 31 - __clz(N);
   float2* z = sz;
-  float2* v = sz + N;
-  float2* tw = sz + 2 * N;
+  float2* v = sz + fft_slot(N) + 1;
+  float2* tw = v + fft_slot(N) + 1;
   twiddles(tw, N);
   const float emax = key_emax(*emax_key);
   const int am = key_argmax(*emax_key);
@@ -917,27 +950,23 @@ __global__ void k_envlog_vjp(Img im, const float* __restrict__ irf, const float*
   const float S = *live_sum;
   for (int l = blockIdx.x; l < im.nl; l += gridDim.x) {
     const float* x = irf + (size_t)l * N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const int j = (int)(__brev((unsigned)i) >> (32 - logN));
-      z[j] = make_float2(__ldg(&x[i]), 0.0f);
-    }
+    for (int i = threadIdx.x; i < N; i += blockDim.x) z[fft_slot(bit_rev(i, logN))] = make_float2(__ldg(&x[i]), 0.0f);
     __syncthreads();
     analytic_smem(z, tw, N, logN);
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const float xi = __ldg(&x[i]), yi = z[i].y;
+      const float xi = __ldg(&x[i]), yi = z[fft_slot(i)].y;
       const float e = sqrtf(xi * xi + yi * yi);
       const int p = l * N + i;
       float ge = 0.0f;
       if (emax > 0.0f && e > 0.0f && 20.0f * log10f(e / emax) > -im.dr) ge = gb[p] * c / e;
       if (p == am && emax > 0.0f) ge -= c * S / emax;
       const float vv = e > 0.0f ? yi / e * ge : 0.0f;
-      z[i] = make_float2(e > 0.0f ? xi / e * ge : 0.0f, 0.0f);  // keep (x/E) g_E in z.x
-      const int j = (int)(__brev((unsigned)i) >> (32 - logN));
-      v[j] = make_float2(vv, 0.0f);
+      z[fft_slot(i)] = make_float2(e > 0.0f ? xi / e * ge : 0.0f, 0.0f);  // keep (x/E) g_E in z.x
+      v[fft_slot(bit_rev(i, logN))] = make_float2(vv, 0.0f);
     }
     __syncthreads();
     analytic_smem(v, tw, N, logN);
-    for (int i = threadIdx.x; i < N; i += blockDim.x) gi[(size_t)l * N + i] = z[i].x - v[i].y;
+    for (int i = threadIdx.x; i < N; i += blockDim.x) gi[(size_t)l * N + i] = z[fft_slot(i)].x - v[fft_slot(i)].y;
     __syncthreads();
   }
 }
@@ -1051,7 +1080,7 @@ void launch_das_adj(const Acq& q, const Img& im, const float* gi, float* grf, in
   }
   k_das_adj_finish<<<grid, 256, 0, st>>>(acc, n, npx, maxbits, grf);
 }
-constexpr int FUSED_SMEM_MAX = 200 * 1024;
+constexpr int FUSED_SMEM_MAX = 202 * 1024;
 static std::atomic<int> g_envlog_fused{1};
 
 }  // namespace usrt
@@ -1072,7 +1101,7 @@ int launch_envlog(const Img& im, const float* irf, float* env, unsigned long lon
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t base = sizeof(float2) * (size_t)(im.nd + im.nd / 2);
+    const size_t base = fft_line_bytes(im.nd) + sizeof(float2) * (size_t)(im.nd / 2);
     for (int lpb = 1; lpb <= 8; ++lpb) {
       const size_t smem = base + sizeof(float) * (size_t)lpb * im.nd;
       if (smem > (size_t)FUSED_SMEM_MAX) break;
@@ -1098,7 +1127,7 @@ int launch_envlog(const Img& im, const float* irf, float* env, unsigned long lon
   if (err == cudaSuccess) {
     void* args[] = {(void*)&im, (void*)&irf, (void*)&env, (void*)&key};
     err = cudaLaunchKernel((const void*)k_envelope, dim3(nb), dim3(256), args,
-                           sizeof(float2) * (size_t)(im.nd + im.nd / 2), st);
+                           fft_line_bytes(im.nd) + sizeof(float2) * (size_t)(im.nd / 2), st);
     launched += err == cudaSuccess;
   }
   if (bmode && err == cudaSuccess) {
@@ -1121,7 +1150,7 @@ void launch_envlog_vjp(const Img& im, const float* irf, const float* gb, float* 
   k_live_sum<<<nparts, 256, 0, st>>>(im, env, key, gb, part);
   k_sum_final<<<1, 1024, 0, st>>>(part, nparts, 1.0f, live_sum);
   const int nb = min(im.nl, grid);
-  k_envlog_vjp<<<nb, 256, sizeof(float2) * (size_t)(2 * im.nd + im.nd / 2), st>>>(im, irf, gb, key, live_sum, gi);
+  k_envlog_vjp<<<nb, 256, 2 * fft_line_bytes(im.nd) + sizeof(float2) * (size_t)(im.nd / 2), st>>>(im, irf, gb, key, live_sum, gi);
 }
 cudaError_t image_set_attrs(int nd) {
   cudaError_t ea = cudaFuncSetAttribute(k_das_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, DT_SMEM_MAX);
@@ -1139,10 +1168,10 @@ cudaError_t image_set_attrs(int nd) {
   e = cudaFuncSetAttribute(k_das_acq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)das_acq_smem(MAX_TX));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_envelope, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(float2) * (size_t)(nd + nd / 2)));
+                                       (int)(fft_line_bytes(nd) + sizeof(float2) * (size_t)(nd / 2)));
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_envlog_vjp, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(sizeof(float2) * (size_t)(2 * nd + nd / 2)));
+                              (int)(2 * fft_line_bytes(nd) + sizeof(float2) * (size_t)(nd / 2)));
 }
 
 }  // namespace usrt
