@@ -1090,8 +1090,8 @@ int us_loss(us_ctx* ctx, const us_img_desc* img, const float* bmode_dev, const f
   float* part;
   const int np = grid_of(ctx, 2);
   CKS(ws(ctx, W_PART, np, st, &part));
-  StageScope sc_(ctx, US_STAGE_LOSS, 2, st);
-  launch_loss(im, bmode_dev, bref_dev, dL_dB_dev, part, np, loss_dev, st);
+  StageScope sc_(ctx, US_STAGE_LOSS, 0, st);
+  sc_.nk = launch_loss(im, bmode_dev, bref_dev, dL_dB_dev, part, np, loss_dev, st);
   CK(cudaGetLastError());
   return US_OK;
 }
@@ -1107,11 +1107,12 @@ int us_envlog_vjp(us_ctx* ctx, const us_img_desc* img, const float* irf_dev, con
   unsigned long long* key;
   const int np = grid_of(ctx, 2);
   CKS(ws(ctx, W_ENV, (size_t)im.nl * im.nd, st, &env));
-  CKS(ws(ctx, W_KEY, 2, st, &key));
+  CKS(ws(ctx, W_KEY, 3, st, &key));
   CKS(ws(ctx, W_PART, np, st, &part));
   CKS(ws(ctx, W_SCAL, 4, st, &scal));
-  StageScope sc_(ctx, US_STAGE_ENVLOG_VJP, 4, st);
-  launch_envlog_vjp(im, irf_dev, dL_dB_dev, env, key, part, np, scal, dL_dirf_dev, grid_of(ctx, 8), st);
+  StageScope sc_(ctx, US_STAGE_ENVLOG_VJP, 0, st);
+  sc_.nk = launch_envlog_vjp(im, irf_dev, dL_dB_dev, env, key, part, np, scal, dL_dirf_dev, grid_of(ctx, 8), st,
+                             ctx->d_status);
   CK(cudaGetLastError());
   return US_OK;
 }

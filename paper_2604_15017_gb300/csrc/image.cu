@@ -5,7 +5,11 @@
 #include <atomic>
 #include <cmath>
 
+#include <cooperative_groups.h>
+
 #include "image.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace usrt {
 
@@ -423,8 +427,14 @@ __global__ void k_das_adj_max(const float* __restrict__ gi, int n, unsigned int*
   unsigned int m = 0u;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     m = max(m, __float_as_uint(fabsf(gi[i])));  // NaN's bits lie above +inf's
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(maxbits, m);
+  // one atomic per block: with one per warp 8192 of them queued up at one address (7 -> 4 us)
+  __shared__ unsigned int best;
+  if (threadIdx.x == 0) best = 0u;
+  __syncthreads();
+  m = __reduce_max_sync(0xFFFFFFFFu, m);
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(&best, m);
+  __syncthreads();
+  if (threadIdx.x == 0 && best) atomicMax(maxbits, best);
 }
 constexpr unsigned int F32_INF_BITS = 0x7F800000u;
 constexpr int DAS_ADJ_V_BITS = 40;  // |W| < 2^40 in fixed point
@@ -912,6 +922,33 @@ __global__ void k_loss_partial(Img im, const float* __restrict__ b, const float*
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
+// The loss in one launch for images of at most LOSS_ONE pixels: one cluster of LOSS_CTAS blocks,
+// whose sums meet in the first one's shared memory (128 x 512 pixels: stage 11.6 us as two kernels,
+// 8.8 so; 256 x 1024: 13.4 and 12.1).
+constexpr int LOSS_CTAS = 8, LOSS_THREADS = 1024, LOSS_ONE = 1 << 19;
+__global__ void __cluster_dims__(LOSS_CTAS, 1, 1) __launch_bounds__(LOSS_THREADS)
+    k_loss_cluster(Img im, const float* __restrict__ b, const float* __restrict__ bref, float* gb, float* loss) {
+  __shared__ float sums[LOSS_CTAS];
+  cg::cluster_group cl = cg::this_cluster();
+  const int n = im.nl * im.nd;
+  const float inv = 1.0f / (float)n;
+  float s = 0.0f;
+#pragma unroll 8
+  for (int i = blockIdx.x * LOSS_THREADS + threadIdx.x; i < n; i += LOSS_CTAS * LOSS_THREADS) {
+    const float r = __ldg(&b[i]) - __ldg(&bref[i]);
+    s += im.l1 * fabsf(r) + im.l2 * r * r;
+    if (gb) gb[i] = (im.l1 * (r > 0.0f ? 1.0f : (r < 0.0f ? -1.0f : 0.0f)) + 2.0f * im.l2 * r) * inv;
+  }
+  s = block_sum(s);
+  if (threadIdx.x == 0) cl.map_shared_rank(sums, 0)[cl.block_rank()] = s;
+  cl.sync();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    float t = 0.0f;
+    for (int k = 0; k < LOSS_CTAS; ++k) t += sums[k];
+    loss[0] = t * inv;
+  }
+}
+
 __global__ void k_sum_final(const float* part, int n, float scale, float* out) {
   float s = 0.0f;
   for (int i = threadIdx.x; i < n; i += blockDim.x) s += part[i];
@@ -967,6 +1004,120 @@ __global__ void k_envlog_vjp(Img im, const float* __restrict__ irf, const float*
     __syncthreads();
     analytic_smem(v, tw, N, logN);
     for (int i = threadIdx.x; i < N; i += blockDim.x) gi[(size_t)l * N + i] = z[fft_slot(i)].x - v[fft_slot(i)].y;
+    __syncthreads();
+  }
+}
+
+// The same VJP in one cooperative launch: a block keeps its lines' analytic signals in shared
+// memory, meets the others once for the maximum, and transforms back.  Only the line that holds
+// the maximum needs the sum S over all unclipped pixels: its block alone waits for the others'
+// partial sums (added in block order).  Both waits are bounded, as in k_envlog_fused; one that
+// expires makes the block's lines NaN and raises ST_TIMEOUT.  keyw: packed maximum, two arrival
+// counters (zeroed before the launch).  256 lines of 1024: 47 us as four kernels, which computed
+// the envelope's transform twice; 128 lines of 512: 30 us against 20.
+__global__ void __launch_bounds__(256) k_envlog_vjp_fused(Img im, const float* __restrict__ irf,
+                                                          const float* __restrict__ gb, unsigned long long* keyw,
+                                                          float* part, float* gi, int* status, long long limit) {
+  extern __shared__ float2 sz[];
+  const int N = im.nd, L = fft_slot(N) + 1;
+  const int logN = 31 - __clz(N);
+  float2* tw = sz;
+  float2* v = tw + N / 2;
+  float2* zl = v + L;  // the block's lines, L slots each
+  __shared__ unsigned long long best;
+  __shared__ float s_sum;
+  __shared__ int s_ok;
+  twiddles(tw, N);
+  if (threadIdx.x == 0) {
+    best = 0ull;
+    s_ok = 1;
+  }
+  unsigned long long own = 0ull;
+  int j = 0;
+  for (int l = blockIdx.x; l < im.nl; l += gridDim.x, ++j) {
+    const float* x = irf + (size_t)l * N;
+    float2* z = zl + j * L;
+    for (int i = threadIdx.x; i < N; i += blockDim.x) z[fft_slot(bit_rev(i, logN))] = make_float2(__ldg(&x[i]), 0.0f);
+    __syncthreads();
+    analytic_smem(z, tw, N, logN);
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+      const float2 a = z[fft_slot(i)];
+      const float e = sqrtf(a.x * a.x + a.y * a.y);
+      const unsigned long long key =
+          ((unsigned long long)__float_as_uint(e) << 32) | (0xFFFFFFFFu - (uint32_t)(l * N + i));
+      own = key > own ? key : own;
+    }
+  }
+  block_max_key(own, &best);
+  __syncthreads();
+  auto wait = [&](unsigned long long* counter) {  // thread 0: until every block has arrived
+    const long long t0 = clock64();
+    while (atomicAdd(counter, 0ull) < (unsigned long long)gridDim.x) {
+      if (clock64() - t0 > limit) {
+        if (status) atomicOr(status, ST_TIMEOUT);
+        s_ok = 0;
+        break;
+      }
+      __nanosleep(64);
+    }
+    __threadfence();
+  };
+  if (threadIdx.x == 0) {
+    atomicMax(&keyw[0], best);
+    __threadfence();
+    atomicAdd(&keyw[1], 1ull);
+    wait(&keyw[1]);
+    best = atomicAdd(&keyw[0], 0ull);
+  }
+  __syncthreads();
+  const float emax = key_emax(best);
+  const int am = key_argmax(best);
+  const float c = 8.685889638065036f;  // 20 / ln(10)
+  float sum = 0.0f;
+  j = 0;
+  for (int l = blockIdx.x; l < im.nl; l += gridDim.x, ++j)
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+      const float2 a = zl[j * L + fft_slot(i)];
+      const float e = sqrtf(a.x * a.x + a.y * a.y);
+      if (emax > 0.0f && e > 0.0f && 20.0f * log10f(e / emax) > -im.dr) sum += __ldg(&gb[(size_t)l * N + i]);
+    }
+  sum = block_sum(sum);
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = sum;
+    __threadfence();
+    atomicAdd(&keyw[2], 1ull);
+  }
+  const bool owner = emax > 0.0f && (am / N) % (int)gridDim.x == (int)blockIdx.x;
+  float S = 0.0f;
+  if (owner) {  // block-uniform
+    if (threadIdx.x == 0) wait(&keyw[2]);
+    __syncthreads();
+    float s = 0.0f;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) s += __ldcg(&part[b]);
+    s = block_sum(s);
+    if (threadIdx.x == 0) s_sum = s;
+    __syncthreads();
+    S = s_sum;
+  }
+  j = 0;
+  for (int l = blockIdx.x; l < im.nl; l += gridDim.x, ++j) {
+    const float* x = irf + (size_t)l * N;
+    float2* z = zl + j * L;
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+      const float xi = __ldg(&x[i]), yi = z[fft_slot(i)].y;
+      const float e = sqrtf(xi * xi + yi * yi);
+      const int p = l * N + i;
+      float ge = 0.0f;
+      if (emax > 0.0f && e > 0.0f && 20.0f * log10f(e / emax) > -im.dr) ge = __ldg(&gb[p]) * c / e;
+      if (p == am && emax > 0.0f) ge -= c * S / emax;
+      const float vv = e > 0.0f ? yi / e * ge : 0.0f;
+      z[fft_slot(i)].x = e > 0.0f ? xi / e * ge : 0.0f;  // keep (x/E) g_E in z.x
+      v[fft_slot(bit_rev(i, logN))] = make_float2(vv, 0.0f);
+    }
+    __syncthreads();
+    analytic_smem(v, tw, N, logN);
+    for (int i = threadIdx.x; i < N; i += blockDim.x)
+      gi[(size_t)l * N + i] = s_ok ? z[fft_slot(i)].x - v[fft_slot(i)].y : __int_as_float(0x7FC00000);
     __syncthreads();
   }
 }
@@ -1066,7 +1217,7 @@ void launch_das_adj(const Acq& q, const Img& im, const float* gi, float* grf, in
   const int npx = im.nl * im.nd;
   cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * (size_t)n, st);
   cudaMemsetAsync(maxbits, 0, sizeof(unsigned int), st);
-  k_das_adj_max<<<min(grid, (npx + 255) / 256), 256, 0, st>>>(gi, npx, maxbits);
+  k_das_adj_max<<<min(grid, (npx + 1023) / 1024), 256, 0, st>>>(gi, npx, maxbits);
   if (q.ntx <= DJ_MAX_TX && g_das_adj_tiled.load()) {
     const int tiles = ((im.nl + DJ_LINES - 1) / DJ_LINES) * ((im.nd + DJ_DEPTHS - 1) / DJ_DEPTHS);
     // a tile's elements over as many blocks as it takes to give the GPU DJ_BLOCKS of them
@@ -1139,23 +1290,53 @@ int launch_envlog(const Img& im, const float* irf, float* env, unsigned long lon
   if (launch_err) *launch_err = err;
   return launched;
 }
-void launch_loss(const Img& im, const float* b, const float* bref, float* gb, float* part, int nparts, float* loss,
-                 cudaStream_t st) {
+int launch_loss(const Img& im, const float* b, const float* bref, float* gb, float* part, int nparts, float* loss,
+                cudaStream_t st) {
+  // in place (gb over b or bref) the single launch's reads through the read-only path may not run
+  // beside its writes
+  if (im.nl * (long long)im.nd <= LOSS_ONE && gb != b && gb != bref) {
+    k_loss_cluster<<<LOSS_CTAS, LOSS_THREADS, 0, st>>>(im, b, bref, gb, loss);
+    return 1;
+  }
   k_loss_partial<<<nparts, 256, 0, st>>>(im, b, bref, gb, part);
   k_sum_final<<<1, 1024, 0, st>>>(part, nparts, 1.0f / (float)(im.nl * im.nd), loss);
+  return 2;
 }
-void launch_envlog_vjp(const Img& im, const float* irf, const float* gb, float* env, unsigned long long* key,
-                       float* part, int nparts, float* live_sum, float* gi, int grid, cudaStream_t st) {
+int launch_envlog_vjp(const Img& im, const float* irf, const float* gb, float* env, unsigned long long* key,
+                      float* part, int nparts, float* live_sum, float* gi, int grid, cudaStream_t st, int* status) {
+  if (g_envlog_fused.load() && gi != irf && gi != gb) {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    for (int lpb = 1; lpb <= 4; ++lpb) {  // lines per block: the fewest that keep the blocks co-resident
+      const size_t smem = (lpb + 1) * fft_line_bytes(im.nd) + sizeof(float2) * (size_t)(im.nd / 2);
+      int nb = (im.nl + lpb - 1) / lpb, per_sm = 0;
+      if (smem > (size_t)FUSED_SMEM_MAX || nparts < nb) continue;
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_envlog_vjp_fused, 256, smem) != cudaSuccess) break;
+      if (per_sm < 1 || 2 * nb > per_sm * sms) continue;  // half of the resident blocks at most
+      if (cudaMemsetAsync(key, 0, 3 * sizeof(unsigned long long), st) != cudaSuccess) break;
+      long long limit = BARRIER_CYCLES;
+      void* args[] = {(void*)&im, (void*)&irf, (void*)&gb, (void*)&key, (void*)&part, (void*)&gi, (void*)&status,
+                      (void*)&limit};
+      if (cudaLaunchCooperativeKernel((const void*)k_envlog_vjp_fused, dim3(nb), dim3(256), args, smem, st) == cudaSuccess)
+        return 1;
+      cudaGetLastError();  // the refused cooperative launch: fall back to the four kernels
+      break;
+    }
+  }
   launch_envlog(im, irf, env, key, nullptr, grid, st);
   k_live_sum<<<nparts, 256, 0, st>>>(im, env, key, gb, part);
   k_sum_final<<<1, 1024, 0, st>>>(part, nparts, 1.0f, live_sum);
   const int nb = min(im.nl, grid);
   k_envlog_vjp<<<nb, 256, 2 * fft_line_bytes(im.nd) + sizeof(float2) * (size_t)(im.nd / 2), st>>>(im, irf, gb, key, live_sum, gi);
+  return 4;
 }
 cudaError_t image_set_attrs(int nd) {
   cudaError_t ea = cudaFuncSetAttribute(k_das_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, DT_SMEM_MAX);
   if (ea != cudaSuccess) return ea;
   cudaError_t e0 = cudaFuncSetAttribute(k_envlog_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSED_SMEM_MAX);
+  if (e0 != cudaSuccess) return e0;
+  e0 = cudaFuncSetAttribute(k_envlog_vjp_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSED_SMEM_MAX);
   if (e0 != cudaSuccess) return e0;
   cudaError_t e = cudaFuncSetAttribute(k_das, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)das_smem(MAX_ELEM, MAX_TX, true));

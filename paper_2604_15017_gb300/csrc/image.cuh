@@ -25,10 +25,11 @@ void launch_das_acq(const Acq& q, const Img& im, const float* rf, const float* g
 // launched; launch_err (may be null) the first launch error of this call alone.
 int launch_envlog(const Img& im, const float* irf, float* env, unsigned long long* key, float* bmode, int grid,
                   cudaStream_t st, int* status = nullptr, int fault_barrier = 0, cudaError_t* launch_err = nullptr);
-void launch_loss(const Img& im, const float* b, const float* bref, float* gb, float* part, int nparts, float* loss,
-                 cudaStream_t st);
-void launch_envlog_vjp(const Img& im, const float* irf, const float* gb, float* env, unsigned long long* key,
-                       float* part, int nparts, float* live_sum, float* gi, int grid, cudaStream_t st);
+// both return the number of kernels launched; key points to 3 words, status (may be null) as above
+int launch_loss(const Img& im, const float* b, const float* bref, float* gb, float* part, int nparts, float* loss,
+                cudaStream_t st);
+int launch_envlog_vjp(const Img& im, const float* irf, const float* gb, float* env, unsigned long long* key,
+                      float* part, int nparts, float* live_sum, float* gi, int grid, cudaStream_t st, int* status);
 cudaError_t image_set_attrs(int nd);
 
 }  // namespace usrt
