@@ -81,9 +81,10 @@ struct Lane {
   cudaStream_t stream = nullptr;  // lane 0: none (the caller's stream)
   cudaEvent_t ev_done = nullptr;
   // second stream for the secondary rays (US_OPT_NEE_STREAM): fork events per round, a join event
-  cudaStream_t side = nullptr;
+  // (a pass without job sorts alternates between two, so that its rounds' kernels overlap)
+  cudaStream_t side = nullptr, side2 = nullptr;
   cudaEvent_t ev_fork[MAX_KMAX + 2] = {};
-  cudaEvent_t ev_join = nullptr;
+  cudaEvent_t ev_join = nullptr, ev_join2 = nullptr;
   cudaEvent_t ev_afork = nullptr, ev_ajoin = nullptr;  // the adjoint's fork and join
 };
 
@@ -215,9 +216,11 @@ void free_lane(us_ctx* ctx, Lane* l) {
   for (cudaEvent_t e : l->ev_fork)
     if (e) cudaEventDestroy(e);
   if (l->ev_join) cudaEventDestroy(l->ev_join);
+  if (l->ev_join2) cudaEventDestroy(l->ev_join2);
   if (l->ev_afork) cudaEventDestroy(l->ev_afork);
   if (l->ev_ajoin) cudaEventDestroy(l->ev_ajoin);
   if (l->side) cudaStreamDestroy(l->side);
+  if (l->side2) cudaStreamDestroy(l->side2);
   if (l->stream) cudaStreamDestroy(l->stream);
   delete l;
 }
@@ -430,6 +433,8 @@ int ensure_side(us_ctx* ctx, Lane* L) {
   CK(cudaStreamCreateWithFlags(&L->side, cudaStreamNonBlocking));
   for (cudaEvent_t& e : L->ev_fork) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&L->ev_join, cudaEventDisableTiming));
+  CK(cudaStreamCreateWithFlags(&L->side2, cudaStreamNonBlocking));
+  CK(cudaEventCreateWithFlags(&L->ev_join2, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&L->ev_afork, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&L->ev_ajoin, cudaEventDisableTiming));
   return US_OK;
@@ -499,6 +504,11 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
   const bool side = do_nee && any_jobs && nee_pct > 0;
   Lane* L = ctx->L;
   if (side) CKS(ensure_side(ctx, L));
+  // unsorted rounds share no scratch: odd ones take another stream, so that a round's secondary rays
+  // need not wait for the previous round's (inverse-problem iteration 1017 -> 950 us, medium render
+  // 1068 -> 1035); only for single calls: with the batch's lanes it made more streams than the
+  // device has queues for (batch of 8 +3.5 %)
+  const bool two_sides = side && !A.sort && !L->stream;
   const int nee_grid = side ? std::max(ctx->num_sms, grid_of(ctx, ctx->nee_per_sm) * nee_pct / 100)
                             : grid_of(ctx, ctx->nee_per_sm);
   RaySort rs;
@@ -562,9 +572,9 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
     // the round's secondary rays (job sort, then the kernel): on the second stream from here
     cudaStream_t ns = st;
     if (side) {
+      ns = two_sides && (k & 1) ? L->side2 : L->side;
       CK(cudaEventRecord(L->ev_fork[k], st));
-      CK(cudaStreamWaitEvent(L->side, L->ev_fork[k], 0));
-      ns = L->side;
+      CK(cudaStreamWaitEvent(ns, L->ev_fork[k], 0));
     }
     if (sort_jobs && k < q.kmax) {
       StageScope sc_(ctx, US_STAGE_JOB_SORT, 3, ns);
@@ -579,6 +589,10 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
   if (side) {
     CK(cudaEventRecord(L->ev_join, L->side));
     CK(cudaStreamWaitEvent(st, L->ev_join, 0));
+    if (two_sides && q.kmax > 0) {  // side2 was forked in round 1
+      CK(cudaEventRecord(L->ev_join2, L->side2));
+      CK(cudaStreamWaitEvent(st, L->ev_join2, 0));
+    }
   }
   CK(cudaGetLastError());
   return US_OK;
