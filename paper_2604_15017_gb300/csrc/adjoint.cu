@@ -21,7 +21,7 @@ namespace usrt {
 // (fs^2 sigma))) instead of a sin/cos and an exp per tap; over the <= 96 taps of the support
 // their rounding grows to a few 1e-6 relative.  Bound by the gathers (each lane reads a row of its
 // own): four samples per read where the rows are 16-byte aligned, and five sums combined at the
-// end instead of three weights per tap.  7.9M arrivals on random rows 690 -> 445 us; secondary-ray
+// end instead of three weights per tap.  7.9M arrivals on random rows 690 -> 395 us; secondary-ray
 // adjoint of the inclusion frame 1640 -> 1335 us.
 // ------------------------------------------------------------------------------------------
 __device__ __forceinline__ void splat_adj_gather(const float* __restrict__ g, float t_hi, float t_lo, float a,
@@ -39,15 +39,14 @@ __device__ __forceinline__ void splat_adj_gather(const float* __restrict__ g, fl
   const float inv_sig = 1.0f / P.sig;
   if (lo <= hi) {
     const float dt = 1.0f / P.fs;
-    const int n4 = lo & ~3;  // rows are whole float4s (n_samples is a multiple of 4)
-    const float x0 = ((float)(n4 - n0) - fr) / P.fs;
+    const float x0 = ((float)(lo - n0) - fr) / P.fs;
     float sn, cs;
     sincosf(w * x0, &sn, &cs);
     float E = expf(-x0 * x0 * inv_sig);
     float q = expf(-(2.0f * x0 + dt) * dt * inv_sig);  // E(x0 + dt) / E(x0)
     auto tap = [&](float gn, int n) {
-      const float x = fmaf((float)(n - n4), dt, x0);
-      const float ge = n >= lo && n <= hi ? gn * E : 0.0f;
+      const float x = fmaf((float)(n - lo), dt, x0);
+      const float ge = gn * E;
       const float p = ge * sn, c = ge * cs, px = p * x;
       s0 += p;
       c0 += c;
@@ -60,17 +59,18 @@ __device__ __forceinline__ void splat_adj_gather(const float* __restrict__ g, fl
       E *= q;
       q *= P.env_qq;
     };
-    if (P.vec) {
-      for (int n = n4; n <= hi; n += 4) {
+    int n = lo;
+    if (P.vec) {  // whole float4s between a head and a tail of at most three samples
+      for (; n <= hi && (n & 3); ++n) tap(__ldg(&g[n]), n);
+      for (; n + 3 <= hi; n += 4) {
         const float4 v = __ldg(reinterpret_cast<const float4*>(g + n));
         tap(v.x, n);
         tap(v.y, n + 1);
         tap(v.z, n + 2);
         tap(v.w, n + 3);
       }
-    } else {
-      for (int n = n4; n <= hi; ++n) tap(__ldg(&g[n]), n);
     }
+    for (; n <= hi; ++n) tap(__ldg(&g[n]), n);
   }
   ga = s0;
   gt = a * (2.0f * inv_sig * s1 - w * c0);
