@@ -202,9 +202,8 @@ __global__ void __launch_bounds__(SC_THREADS) k_row_scatter(Src src, const uint3
 // convolution.  The moments of a whole 4096-sample row take 153 KB, one block per SM, whose
 // barriers and dependent passes nothing hid; a segment's take 78 KB, so two blocks of 512 threads
 // share an SM and overlap each other's phases.  A segment re-reduces its halo's arrivals (6 %).
-// The convolution's threads are 256 groups of 8 samples x 2 halves of the moments.  2048 rows of
-// 4096 samples, 7.9M arrivals: 459 -> 342 us (segments of 1024, three blocks: 345, and slower on
-// a hundred rows); 64 nearly empty rows 18.7 -> 16.7 us.
+// 2048 rows of 4096 samples, 7.9M arrivals: 459 -> 320 us (segments of 1024, three blocks: equal,
+// and slower on a hundred rows); 64 nearly empty rows 18.7 -> 16.7 us.
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(ROW_THREADS, 2) k_row_splat(SplatGeom g, const uint2* bucket, const uint32_t* off,
                                                               uint2* scratch, const float* Gtab, float* rf) {
@@ -213,7 +212,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) k_row_splat(SplatGeom g, const
   const int NB = g.nbins;         // bins -HALO .. ns + HALO - 1
   constexpr int MS = row_mom_stride(ROW_SEG);
   const int sh = row_mom_shift(g);  // bin x of a segment is stored at mom_slot(x + sh)
-  float* M = smf;                 // [K_MOM][MS], padded: one spare slot after every 8; then the partial sums
+  float* M = smf;                 // [K_MOM][MS], padded: one spare slot after every 8
   float* G = M + K_MOM * MS;      // [K_MOM][MAX_TAPS], zero past ntaps
   uint32_t* hist = reinterpret_cast<uint32_t*>(G + K_MOM * MAX_TAPS);  // [NB]
   __shared__ uint32_t part[ROW_THREADS / 32];
@@ -314,19 +313,19 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) k_row_splat(SplatGeom g, const
     }
     __syncthreads();
     // convolution: out[n] = sum_j sum_d G_j[d] M_j[bin n - dlo - d]; a thread produces 8 consecutive
-    // samples from two of the moments.  Taps go in blocks of 8: the 15 moments a block touches are
-    // read once into registers (a sliding window) and feed 64 FMAs.  The shift sh puts every
-    // window start on a multiple of 8, so the padded slots of the window are fixed offsets and
-    // the lanes of a warp read addresses 9 apart: no bank conflicts.
-    constexpr int GROUPS = ROW_SEG / 8, JG = ROW_THREADS / GROUPS;
-    const int n0 = 8 * (tid % GROUPS), jg = tid / GROUPS;
-    float acc[8];
-#pragma unroll
-    for (int r = 0; r < 8; ++r) acc[r] = 0.0f;
+    // samples (the half of the block that has none waits: the other block's warps fill the SM).
+    // Taps go in blocks of 8: the 15 moments a block touches are read once into registers (a
+    // sliding window) and feed 64 FMAs.  The shift sh puts every window start on a multiple of 8,
+    // so the padded slots of the window are fixed offsets and the lanes of a warp read addresses
+    // 9 apart: no bank conflicts.
+    const int n0 = 8 * tid;
     if (n0 < n_seg) {
+      float acc[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) acc[r] = 0.0f;
       const int xs0 = n0 - g.dlo + HALO + sh - 7;  // window start for taps 0..7, a multiple of 8
       const int ntp = (g.ntaps + 7) & ~7;
-      for (int j = jg * (K_MOM / JG); j < (jg + 1) * (K_MOM / JG); ++j) {
+      for (int j = 0; j < K_MOM; ++j) {
         const float* Mj = M + j * MS;
         const float* Gj = G + j * MAX_TAPS;
         for (int d0 = 0; d0 < ntp; d0 += 8) {
@@ -342,17 +341,9 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) k_row_splat(SplatGeom g, const
           }
         }
       }
-    }
-    __syncthreads();
-    float* P = M;  // [JG][GROUPS * 9]: the moment groups' sums, one spare slot after every 8
-#pragma unroll
-    for (int r = 0; r < 8; ++r) P[jg * (GROUPS * 9) + (n0 / 8) * 9 + r] = acc[r];
-    __syncthreads();
-    for (int n = tid; n < n_seg; n += ROW_THREADS) {
-      float v = 0.0f;
-#pragma unroll
-      for (int k = 0; k < JG; ++k) v += P[k * (GROUPS * 9) + mom_slot(n)];
-      out_row[s0 + n] = v;
+      float* out = out_row + s0 + n0;  // rows, segments and groups are whole float4s; rf is 16-byte aligned
+      reinterpret_cast<float4*>(out)[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+      if (n0 + 4 < n_seg) reinterpret_cast<float4*>(out)[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
     }
     __syncthreads();
   }
