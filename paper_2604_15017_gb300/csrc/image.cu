@@ -1231,6 +1231,30 @@ void launch_das_adj(const Acq& q, const Img& im, const float* gi, float* grf, in
   }
   k_das_adj_finish<<<grid, 256, 0, st>>>(acc, n, npx, maxbits, grf);
 }
+// resident blocks on the current device (all SMs) of a kernel of 256 threads with `smem` bytes, asked
+// of the runtime once per device, kernel and size: the answer never changes, and a query costs as
+// much host time as a launch
+static int resident_blocks(const void* kernel, size_t smem) {
+  struct Entry {
+    int dev;
+    const void* kernel;
+    size_t smem;
+    int blocks;
+  };
+  constexpr int SLOTS = 32;
+  static thread_local Entry seen[SLOTS];
+  static thread_local int used = 0;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  for (int k = 0; k < std::min(used, SLOTS); ++k)
+    if (seen[k].dev == dev && seen[k].kernel == kernel && seen[k].smem == smem) return seen[k].blocks;
+  int per_sm = 0, sms = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 256, smem) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 0;
+  seen[used++ % SLOTS] = Entry{dev, kernel, smem, per_sm * sms};
+  return per_sm * sms;
+}
 constexpr int FUSED_SMEM_MAX = 202 * 1024;
 static std::atomic<int> g_envlog_fused{1};
 
@@ -1249,17 +1273,13 @@ int launch_envlog(const Img& im, const float* irf, float* env, unsigned long lon
   int launched = 0;
   if (bmode && g_envlog_fused.load() && err == cudaSuccess) {
     // fused path: every line's envelope stays in the shared memory of a co-resident block
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t base = fft_line_bytes(im.nd) + sizeof(float2) * (size_t)(im.nd / 2);
     for (int lpb = 1; lpb <= 8; ++lpb) {
       const size_t smem = base + sizeof(float) * (size_t)lpb * im.nd;
       if (smem > (size_t)FUSED_SMEM_MAX) break;
-      int per_sm = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_envlog_fused, 256, smem) != cudaSuccess) break;
+      const int resident = resident_blocks((const void*)k_envlog_fused, smem);
       const int nb = (im.nl + lpb - 1) / lpb;
-      if (per_sm > 0 && nb <= per_sm * sms) {
+      if (resident > 0 && nb <= resident) {
         int extra = fault_barrier ? 1 : 0;
         long long limit = fault_barrier ? FAULT_BARRIER_CYCLES : BARRIER_CYCLES;
         void* args[] = {(void*)&im, (void*)&irf, (void*)&key, (void*)&bmode, (void*)&status, (void*)&extra,
@@ -1305,15 +1325,12 @@ int launch_loss(const Img& im, const float* b, const float* bref, float* gb, flo
 int launch_envlog_vjp(const Img& im, const float* irf, const float* gb, float* env, unsigned long long* key,
                       float* part, int nparts, float* live_sum, float* gi, int grid, cudaStream_t st, int* status) {
   if (g_envlog_fused.load() && gi != irf && gi != gb) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     for (int lpb = 1; lpb <= 4; ++lpb) {  // lines per block: the fewest that keep the blocks co-resident
       const size_t smem = (lpb + 1) * fft_line_bytes(im.nd) + sizeof(float2) * (size_t)(im.nd / 2);
-      int nb = (im.nl + lpb - 1) / lpb, per_sm = 0;
+      const int nb = (im.nl + lpb - 1) / lpb;
       if (smem > (size_t)FUSED_SMEM_MAX || nparts < nb) continue;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_envlog_vjp_fused, 256, smem) != cudaSuccess) break;
-      if (per_sm < 1 || 2 * nb > per_sm * sms) continue;  // half of the resident blocks at most
+      // half of the resident blocks at most
+      if (2 * nb > resident_blocks((const void*)k_envlog_vjp_fused, smem)) continue;
       if (cudaMemsetAsync(key, 0, 3 * sizeof(unsigned long long), st) != cudaSuccess) break;
       long long limit = BARRIER_CYCLES;
       void* args[] = {(void*)&im, (void*)&irf, (void*)&gb, (void*)&key, (void*)&part, (void*)&gi, (void*)&status,
