@@ -73,6 +73,35 @@ __device__ __forceinline__ ff das_urx(const DasRx& p, ff xe) {
   const float res = __fadd_rn(__fmaf_rn(-r, r, r2), __fadd_rn(s.lo, __fadd_rn(l, p.z2.lo)));
   return ff{r, __fmul_rn(res, __fmul_rn(0.5f, inv))};
 }
+// the same for two elements at once (their negated positions side by side), operation by operation in
+// packed FP32: the same bits, half the issue slots
+struct DasRx2 {
+  f32x2 xh, xl, zh, zl;
+};
+__device__ __forceinline__ DasRx2 das_rx2(const DasRx& p) {
+  return DasRx2{pack2(p.x.hi, p.x.hi), pack2(p.x.lo, p.x.lo), pack2(p.z2.hi, p.z2.hi), pack2(p.z2.lo, p.z2.lo)};
+}
+__device__ __forceinline__ f32x2 two_sum2(f32x2 a, f32x2 b, f32x2& e) {
+  const f32x2 s = add2(a, b), bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+  return s;
+}
+__device__ __forceinline__ void das_urx2(const DasRx2& p, f32x2 nxh, f32x2 nxl, ff& u0, ff& u1) {
+  f32x2 e, e2;
+  const f32x2 s = two_sum2(p.xh, nxh, e);
+  const f32x2 t = add2(e, add2(p.xl, nxl));
+  const f32x2 dh = add2(s, t), dl = sub2(t, sub2(dh, s));
+  const f32x2 h = mul2(dh, dh);
+  const f32x2 l = fma2(add2(dh, dh), dl, fma2(dh, dh, neg2(h)));
+  const float2 sh = unpack2(two_sum2(h, p.zh, e2));
+  const float ra = fmaxf(sh.x, 1e-30f), rb = fmaxf(sh.y, 1e-30f);
+  const f32x2 r2 = pack2(ra, rb), inv = pack2(rsqrtf(ra), rsqrtf(rb));
+  const f32x2 r = mul2(r2, inv);
+  const f32x2 res = add2(fma2(neg2(r), r, r2), add2(e2, add2(l, p.zl)));
+  const float2 hi = unpack2(r), lo = unpack2(mul2(res, mul2(pack2(0.5f, 0.5f), inv)));
+  u0 = ff{hi.x, lo.x};
+  u1 = ff{hi.y, lo.y};
+}
 __device__ __forceinline__ float hann_w(int e, int ne) {
   return 0.5f * (1.0f - cospif(2.0f * (float)(e + 1) / (float)(ne + 1)));
 }
@@ -121,22 +150,26 @@ __device__ __forceinline__ void das_tap(float2 a, float2 b, int& i, float& f) {
 // the pixel's smallest and largest transmit delay.  The elements of a chunk are shared out over
 // DAS_ES groups of threads, so that small images fill the GPU too; a pixel's sums over the
 // transmits meet in shared memory and are weighted and added in element order by one thread.
-// 128 elements, 256 x 1024 pixels: 16 transmits 921 -> 378 us (5.4e8 taps), 1 transmit 239 ->
-// 133 us (there the delays, 3.4e7 of them, are most of it).  Elements split two ways instead of four,
-// patches of 16 x 2 and 4 x 8: equal or slower.
+// A thread takes two neighbouring elements at a time: their delays in packed FP32, one read of each
+// transmit delay, four independent gathers in flight.  128 elements, 256 x 1024 pixels: 16
+// transmits 921 us at first, 378 with an element at a time, 341 in pairs (5.4e8 taps); 1 transmit
+// 239, 133, 120 us (there the delays, 3.4e7 of them, are most of it).  Elements split two ways
+// instead of four, patches of 16 x 2 and 4 x 8, more blocks at fewer registers: equal or slower.
 constexpr int DAS_THREADS = 256;
 constexpr int DAS_ES = 4, DAS_TL = 8, DAS_TD = 8, DAS_PX = DAS_TL * DAS_TD;
 constexpr int DAS_EC = 32;  // elements per chunk
-static_assert(DAS_PX * DAS_ES == DAS_THREADS && DAS_TL == 8 && DAS_EC % DAS_ES == 0, "a warp is 8 lines x 4 depths");
+static_assert(DAS_PX * DAS_ES == DAS_THREADS && DAS_TL == 8 && DAS_EC % (2 * DAS_ES) == 0,
+              "a warp is 8 lines x 4 depths, its elements come in pairs");
 __host__ __device__ constexpr size_t das_smem(int ne, int ntx, bool dynamic) {
-  return sizeof(float2) * ((size_t)ntx * DAS_PX + ne) + sizeof(float) * (ne + (dynamic ? 4 : 2) * DAS_EC * DAS_PX);
+  return sizeof(ulonglong2) * ((ne + 1) / 2) + sizeof(float2) * (size_t)ntx * DAS_PX +
+         sizeof(float) * (ne + (dynamic ? 4 : 2) * DAS_EC * DAS_PX);
 }
 __global__ void __launch_bounds__(DAS_THREADS) k_das(Acq q, Img im, const float* __restrict__ rf,
                                                      float* __restrict__ irf) {
-  extern __shared__ float2 das_sm[];
-  float2* utx_s = das_sm;                                     // [ntx][DAS_PX]: (first sample + row offset, fraction)
-  float2* xe_s = das_sm + q.ntx * DAS_PX;                     // [ne] element positions (float-float)
-  float* w_s = reinterpret_cast<float*>(xe_s + q.ne);         // [ne] Hann weights
+  extern __shared__ __align__(16) ulonglong2 das_sm[];
+  ulonglong2* xe_s = das_sm;                                  // [(ne + 1) / 2] negated positions of element pairs
+  float2* utx_s = reinterpret_cast<float2*>(xe_s + (q.ne + 1) / 2);  // [ntx][DAS_PX]: (first sample + row offset, fraction)
+  float* w_s = reinterpret_cast<float*>(utx_s + q.ntx * DAS_PX);     // [ne] Hann weights
   float* s_s = w_s + q.ne;                                    // [2][DAS_EC][DAS_PX] sums over the transmits
   float* wd_s = s_s + 2 * DAS_EC * DAS_PX;                    // the same of the dynamic aperture's weights
   const DasGeo g = das_geo(q);
@@ -151,10 +184,10 @@ __global__ void __launch_bounds__(DAS_THREADS) k_das(Acq q, Img im, const float*
     const float2 u = das_split(das_utx(q, g, x, z, t));
     utx_s[t * DAS_PX + px] = make_float2(__int_as_float(__float_as_int(u.x) + t * tstride), u.y);
   }
-  for (int e = threadIdx.x; e < q.ne; e += DAS_THREADS) {
-    const ff xe = das_elem(q, g, e);
-    xe_s[e] = make_float2(xe.hi, xe.lo);
-    w_s[e] = hann_w(e, q.ne);
+  for (int e = threadIdx.x; e < q.ne; e += DAS_THREADS) w_s[e] = hann_w(e, q.ne);
+  for (int k = threadIdx.x; k < (q.ne + 1) / 2; k += DAS_THREADS) {
+    const ff a = das_elem(q, g, 2 * k), b = das_elem(q, g, min(2 * k + 1, q.ne - 1));
+    xe_s[k] = make_ulonglong2(pack2(-a.hi, -b.hi), pack2(-a.lo, -b.lo));
   }
   __syncthreads();
   int imin = 0x7FFFFFFF, imax = -0x7FFFFFFF;
@@ -166,43 +199,62 @@ __global__ void __launch_bounds__(DAS_THREADS) k_das(Acq q, Img im, const float*
   // clamped so that no sum below overflows, and none of clamped values passes the check
   imin = max(-(1 << 22), min(imin, 1 << 22));
   imax = max(-(1 << 22), min(imax, 1 << 22));
-  const DasRx p = das_rx(g, x, z);
+  const DasRx2 p = das_rx2(das_rx(g, x, z));
   const bool dynamic = im.fnum > 0.0f;
   float acc = 0.0f;
   for (int e0 = 0, buf = 0; e0 < q.ne; e0 += DAS_EC, buf ^= 1) {
     const int e1 = min(e0 + DAS_EC, q.ne);
     float* sb = s_s + buf * DAS_EC * DAS_PX + px;
     float* wb = wd_s + buf * DAS_EC * DAS_PX + px;
-    for (int e = e0 + es; e < e1; e += DAS_ES) {
-      const float2 xe = xe_s[e];
-      const float2 ur = das_split(das_urx(p, ff{xe.x, xe.y}));
-      const int ir = __float_as_int(ur.x);
-      const float2 b = make_float2(__int_as_float(ir + e * q.ns), ur.y);
-      float s = 0.0f;
-      const int irc = max(-(1 << 24), min(ir, 1 << 24));
-      if (irc + imin >= 0 && irc + imax + 2 < q.ns) {  // every tap's two samples lie inside the record
+    for (int e = e0 + 2 * es; e < e1; e += 2 * DAS_ES) {  // elements e and e + 1 (e0 is even)
+      const ulonglong2 xe = xe_s[e >> 1];
+      ff ua, ub;
+      das_urx2(p, xe.x, xe.y, ua, ub);
+      const float2 ra = das_split(ua), rb = das_split(ub);
+      const int ia = __float_as_int(ra.x), ib = __float_as_int(rb.x);
+      const bool two = e + 1 < e1;
+      float sa = 0.0f, sb2 = 0.0f;
+      const int lo = max(-(1 << 24), min(min(ia, ib), 1 << 24)), hi = max(-(1 << 24), min(max(ia, ib), 1 << 24));
+      if (lo + imin >= 0 && hi + imax + 2 < q.ns) {  // every tap's two samples lie inside the record
+        const float2 ba = make_float2(__int_as_float(ia + e * q.ns), ra.y);
+        // past the last element of an odd array the pair's second is the last one again
+        const float2 bb = make_float2(__int_as_float(ib + (two ? e + 1 : e) * q.ns), rb.y);
 #pragma unroll 4
         for (int t = 0; t < q.ntx; ++t) {
-          int i;
-          float f;
-          das_tap(utx_s[t * DAS_PX + px], b, i, f);
-          const float v0 = __ldg(&rf[i]), v1 = __ldg(&rf[i + 1]);
-          s += fmaf(f, v1 - v0, v0);
+          const float2 u = utx_s[t * DAS_PX + px];
+          int i, j;
+          float f, h;
+          das_tap(u, ba, i, f);
+          das_tap(u, bb, j, h);
+          const float v0 = __ldg(&rf[i]), v1 = __ldg(&rf[i + 1]), w0 = __ldg(&rf[j]), w1 = __ldg(&rf[j + 1]);
+          sa += fmaf(f, v1 - v0, v0);
+          sb2 += fmaf(h, w1 - w0, w0);
         }
       } else {
-        for (int t = 0; t < q.ntx; ++t) {
-          int i;
-          float f;
-          das_tap(utx_s[t * DAS_PX + px], b, i, f);
-          const float* row = rf + (size_t)t * tstride + (size_t)e * q.ns;
-          i -= t * tstride + e * q.ns;
-          const float v0 = (i >= 0 && i < q.ns) ? __ldg(&row[i]) : 0.0f;
-          const float v1 = (i + 1 >= 0 && i + 1 < q.ns) ? __ldg(&row[i + 1]) : 0.0f;
-          s += fmaf(f, v1 - v0, v0);
+        for (int k = 0; k < (two ? 2 : 1); ++k) {
+          const float2 b = k ? rb : ra;
+          float s = 0.0f;
+          for (int t = 0; t < q.ntx; ++t) {
+            float2 u = utx_s[t * DAS_PX + px];
+            u.x = __int_as_float(__float_as_int(u.x) - t * tstride);
+            int i;
+            float f;
+            das_tap(u, b, i, f);
+            const float* row = rf + (size_t)t * tstride + (size_t)(e + k) * q.ns;
+            const float v0 = (i >= 0 && i < q.ns) ? __ldg(&row[i]) : 0.0f;
+            const float v1 = (i + 1 >= 0 && i + 1 < q.ns) ? __ldg(&row[i + 1]) : 0.0f;
+            s += fmaf(f, v1 - v0, v0);
+          }
+          if (k) sb2 = s;
+          else sa = s;
         }
       }
-      sb[(e - e0) * DAS_PX] = s;
+      sb[(e - e0) * DAS_PX] = sa;
       if (dynamic) wb[(e - e0) * DAS_PX] = apod_w(q, im, x.hi, z.hi, e);
+      if (two) {
+        sb[(e + 1 - e0) * DAS_PX] = sb2;
+        if (dynamic) wb[(e + 1 - e0) * DAS_PX] = apod_w(q, im, x.hi, z.hi, e + 1);
+      }
     }
     __syncthreads();  // the other buffer is written next; this one again only after the next barrier
     if (es == 0)
