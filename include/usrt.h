@@ -167,7 +167,8 @@ enum {
   /* secondary rays on a second stream: 0 runs each round's secondary-ray kernel after that
    * round's primary rays on the call's stream; p in 1..100 (default 100) runs it on a second
    * stream of the lane (forked and joined with events, so the call stays one stream-ordered
-   * unit), overlapping the next rounds' primary rays, with p % of its resident grid. */
+   * unit), overlapping the next rounds' primary rays, with p % of its resident grid.  Small
+   * passes of a single call, whose jobs are not sorted, alternate between two such streams. */
   US_OPT_NEE_STREAM = 2,
   /* fault injection for tests of the timeout report (default 0): 1 makes the fused envelope
    * kernel's grid barrier wait for one arrival more than there are blocks, with a 1 ms limit,
@@ -186,11 +187,13 @@ int us_set_option(us_ctx* ctx, int option, int value);
  * synchronisation fails. */
 int us_get_status(us_ctx* ctx, int clear, int* device_status);
 
-/* Envelope + log compression kernels, process-wide: enable != 0 (the default) uses the
- * cooperative fused kernel whenever the image's lines fit co-resident blocks; 0 always takes
- * the two-kernel path (envelope, then log compression; the path images too large for the fused
- * kernel take).  Both give the same image.  Applies to every call that forms a B-mode image
- * (us_forward, us_bmode, us_envlog, us_envlog_noalloc); meant for tests of the second path. */
+/* Envelope + log compression kernels and their VJP, process-wide: enable != 0 (the default) uses
+ * the cooperative fused kernel whenever the image's lines fit co-resident blocks; 0 always takes
+ * the path of several kernels (envelope, then log compression; for the VJP also the sum over live
+ * pixels), which images too large for the fused kernels take.  Both give the same image; the VJP
+ * differs only in the order of one sum.  Applies to every call that forms a B-mode image
+ * (us_forward, us_bmode, us_envlog, us_envlog_noalloc) or differentiates one; meant for tests of
+ * the second path. */
 void us_set_envlog_fused(int enable);
 
 /* Transposed DAS kernels, process-wide: enable != 0 (the default) uses the tiled kernel

@@ -189,8 +189,8 @@ def img_desc(img):
 
 
 def set_envlog_fused(enable):
-    """Process-wide: the cooperative fused envelope kernel (True, default) or always the
-    two-kernel path (False)."""
+    """Process-wide: the cooperative fused envelope kernel and its VJP (True, default) or always
+    the path of several kernels (False)."""
     lib().us_set_envlog_fused(int(bool(enable)))
 
 
