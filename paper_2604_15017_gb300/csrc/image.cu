@@ -141,6 +141,18 @@ __device__ __forceinline__ void das_tap(float2 a, float2 b, int& i, float& f) {
   }
 }
 
+// One check for all taps of a pixel and two elements: the extremes of the transmit delays' whole
+// samples (das_tx_range, once per pixel) and the two receive delays'.  Nothing passes where a
+// transmit delay is past 2^22 samples, nor where a receive delay is past 2^24: records are
+// shorter (make_acq), and no sum overflows.
+__device__ __forceinline__ void das_tx_range(int& imin, int& imax) {
+  if (imin < -(1 << 22) || imax > (1 << 22)) imin = -(1 << 28), imax = 0;
+}
+__device__ __forceinline__ bool das_inside(int ia, int ib, int imin, int imax, int ns) {
+  const int lo = max(-(1 << 24), min(min(ia, ib), 1 << 24)), hi = max(-(1 << 24), min(max(ia, ib), 1 << 24));
+  return lo + imin >= 0 && hi + imax + 2 < ns;  // every tap's two samples lie inside the record
+}
+
 // DAS.  A block owns a tile of DAS_TL lines x DAS_TD depths; a warp covers 8 lines x 4 depths.
 // Bound by the L1's gathers: neighbouring depths are ~3 samples apart, neighbouring lines less than
 // one on average, so a warp of 32 depths read 4 lines of 128 bytes per load and 12 bytes per tap
@@ -152,8 +164,8 @@ __device__ __forceinline__ void das_tap(float2 a, float2 b, int& i, float& f) {
 // transmits meet in shared memory and are weighted and added in element order by one thread.
 // A thread takes two neighbouring elements at a time: their delays in packed FP32, one read of each
 // transmit delay, four independent gathers in flight.  128 elements, 256 x 1024 pixels: 16
-// transmits 921 us at first, 378 with an element at a time, 341 in pairs (5.4e8 taps); 1 transmit
-// 239, 133, 120 us (there the delays, 3.4e7 of them, are most of it).  Elements split two ways
+// transmits 921 us at first, 378 with an element at a time, 342 in pairs (5.4e8 taps); 1 transmit
+// 239, 133, 109 us (there the delays, 3.4e7 of them, are most of it).  Elements split two ways
 // instead of four, patches of 16 x 2 and 4 x 8, more blocks at fewer registers: equal or slower.
 constexpr int DAS_THREADS = 256;
 constexpr int DAS_ES = 4, DAS_TL = 8, DAS_TD = 8, DAS_PX = DAS_TL * DAS_TD;
@@ -196,9 +208,7 @@ __global__ void __launch_bounds__(DAS_THREADS) k_das(Acq q, Img im, const float*
     imin = min(imin, i);
     imax = max(imax, i);
   }
-  // clamped so that no sum below overflows, and none of clamped values passes the check
-  imin = max(-(1 << 22), min(imin, 1 << 22));
-  imax = max(-(1 << 22), min(imax, 1 << 22));
+  das_tx_range(imin, imax);
   const DasRx2 p = das_rx2(das_rx(g, x, z));
   const bool dynamic = im.fnum > 0.0f;
   float acc = 0.0f;
@@ -214,8 +224,7 @@ __global__ void __launch_bounds__(DAS_THREADS) k_das(Acq q, Img im, const float*
       const int ia = __float_as_int(ra.x), ib = __float_as_int(rb.x);
       const bool two = e + 1 < e1;
       float sa = 0.0f, sb2 = 0.0f;
-      const int lo = max(-(1 << 24), min(min(ia, ib), 1 << 24)), hi = max(-(1 << 24), min(max(ia, ib), 1 << 24));
-      if (lo + imin >= 0 && hi + imax + 2 < q.ns) {  // every tap's two samples lie inside the record
+      if (das_inside(ia, ib, imin, imax, q.ns)) {
         const float2 ba = make_float2(__int_as_float(ia + e * q.ns), ra.y);
         // past the last element of an odd array the pair's second is the last one again
         const float2 bb = make_float2(__int_as_float(ib + (two ? e + 1 : e) * q.ns), rb.y);

@@ -71,3 +71,21 @@ def test_transposed_das_tiled_equals_untiled(ctx, ne, ntx, ns, nl, nd, depth):
         usrt.set_das_adj_tiled(True)
     assert torch.equal(tiled, plain)
     assert float(tiled.abs().max()) > 0.0
+
+
+def test_das_far_beside_the_array(ctx):
+    """Pixels 4.2e6 samples beside the array under a steering of 88 degrees: the transmit delay falls
+    below -2^22 samples, past which a pixel's taps are not checked all at once, and the sums run
+    across the record's end."""
+    from test_gpu_acq import exact_angles
+
+    degs = [88.0, 87.99]
+    acq = dict(P.acquisition(33, float(np.float32(0.3 * MM)), 2720, degs, 1, 1, 1540.0), angles=exact_angles(degs))
+    img = P.image(9, 32, float(np.float32(-161.66)), float(np.float32(-161.58)), 0.0, float(np.float32(0.03)))
+    rf = np.random.default_rng(5).normal(size=(2, 33, 2720)).astype(np.float32)
+    for k in ("pitch", "c_bf", "fs"):
+        acq[k] = float(np.float32(acq[k]))
+    ref = O.das(acq, img, rf.astype(np.float64))
+    bound = 2e-3 * O.das(acq, img, np.abs(rf).astype(np.float64)) + 1e-6 * np.abs(ref).max()
+    got = ctx.das(acq, img, dev(rf)).cpu().numpy()
+    assert np.all(np.abs(got - ref) <= bound), np.max(np.abs(got - ref) - bound)
