@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
@@ -140,7 +141,6 @@ __device__ __forceinline__ void das_tap(float2 a, float2 b, int& i, float& f) {
     ++i;
   }
 }
-
 // One check for all taps of a pixel and two elements: the extremes of the transmit delays' whole
 // samples (das_tx_range, once per pixel) and the two receive delays'.  Nothing passes where a
 // transmit delay is past 2^22 samples, nor where a receive delay is past 2^24: records are
@@ -1192,55 +1192,119 @@ __global__ void __launch_bounds__(256) k_envlog_vjp_fused(Img im, const float* _
 // 1)/2)) fs / c_bf (transmit aperture and receive distance r); only the transmit delay holds
 // th_t: du/dth = (x cos th - z sin th + W/2 sgn(sin th) cos th) fs / c_bf, sgn(0) = 0.  So a
 // pixel needs, per transmit, S1 = sum_e w_e slope, and over all its taps sum w_e slope u and
-// sum w_e slope du/dp.  One pixel per thread (one pass, no grid stride), elements outer and
-// transmits inner as in k_das, so the receive delay, its pitch derivative and the element
-// weight are evaluated once per (pixel, element); the transmit delays and the per-transmit
-// sums S1 sit in shared memory in thread-major rows; the other two sums are per-pixel scalars
-// (their transmit weights are known before the sum).  Each block writes one
-// row of 2 + ntx sums, reduced in a fixed order (deterministic).
+// sum w_e slope du/dp.  One pixel per thread, a warp 8 lines x 4 depths as in k_das, elements outer
+// (in pairs, their delays in packed FP32) and transmits inner, so the receive delay, its pitch
+// derivative and the element weight are evaluated once per (pixel, element); the transmit delays
+// and the per-transmit sums S1 sit in shared memory in thread-major rows; the other two sums are
+// per-pixel scalars (their transmit weights are known before the sum).  Taps are checked against the
+// record once per pair of elements, for the whole warp: with a check per pixel, warps across the
+// record's end ran both loops.  Each block writes one row of 2 + ntx sums, reduced in a fixed order
+// (deterministic).  Bound by issue and by the gathers' latency.  128 elements, 11 transmits, 96 x
+// 512 pixels 377 -> 200 us; 95 elements, 6 transmits, 101 x 1024 pixels, a third of the taps past
+// the record 188 -> 157 us (170 with a check per pixel, 164 with one per tap).
 // ------------------------------------------------------------------------------------------
 constexpr int DA_THREADS = 256;
-__host__ __device__ constexpr size_t das_acq_smem(int ntx) { return (sizeof(float2) + sizeof(float)) * DA_THREADS * ntx; }
+constexpr int DA_TL = 8, DA_TD = 32;  // a block's lines x depths; a warp has 8 lines x 4 depths
+static_assert(DA_TL * DA_TD == DA_THREADS, "a pixel per thread");
+__host__ __device__ constexpr size_t das_acq_smem(int ne, int ntx) {
+  return sizeof(ulonglong2) * ((ne + 1) / 2) + (sizeof(float2) + sizeof(float)) * DA_THREADS * ntx + sizeof(float) * ne;
+}
 __global__ void __launch_bounds__(DA_THREADS) k_das_acq(Acq q, Img im, const float* __restrict__ rf,
                                                         const float* __restrict__ gi, float* part) {
-  extern __shared__ float2 da_sm[];
-  float2* ut_s = da_sm;                                              // [ntx][DA_THREADS]
-  float* s1_s = reinterpret_cast<float*>(da_sm + q.ntx * DA_THREADS);  // [ntx][DA_THREADS]
-  const int npx = im.nl * im.nd;
+  extern __shared__ __align__(16) ulonglong2 da_sm[];
+  ulonglong2* xe_s = da_sm;                                            // [(ne + 1) / 2] as in k_das
+  float2* ut_s = reinterpret_cast<float2*>(xe_s + (q.ne + 1) / 2);     // [ntx][DA_THREADS]
+  float* s1_s = reinterpret_cast<float*>(ut_s + q.ntx * DA_THREADS);   // [ntx][DA_THREADS]
+  float* w_s = s1_s + q.ntx * DA_THREADS;                              // [ne] Hann weights
   const DasGeo g = das_geo(q);
-  const int p = blockIdx.x * DA_THREADS + threadIdx.x;
-  const bool valid = p < npx;
-  const int l = valid ? p / im.nd : 0, d = valid ? p - l * im.nd : 0;
-  const ff x = grid_coord(im.x0, im.x1, l, im.nl), z = grid_coord(im.z0, im.z1, d, im.nd);
-  const float gp = valid ? __ldg(&gi[p]) : 0.0f;
+  const int tiles_d = (im.nd + DA_TD - 1) / DA_TD;
+  const int tl = blockIdx.x / tiles_d, td = blockIdx.x - tl * tiles_d;
+  const int l = tl * DA_TL + (threadIdx.x & 7), d = td * DA_TD + (threadIdx.x >> 3);
+  const bool valid = l < im.nl && d < im.nd;
+  const ff x = grid_coord(im.x0, im.x1, valid ? l : 0, im.nl), z = grid_coord(im.z0, im.z1, valid ? d : 0, im.nd);
+  const float gp = valid ? __ldg(&gi[(size_t)l * im.nd + d]) : 0.0f;
   const float kfs = q.fs / q.cbf, hn = 0.5f * (float)(q.ne - 1), hw = hn * q.pitch;
+  for (int e = threadIdx.x; e < q.ne; e += DA_THREADS) w_s[e] = hann_w(e, q.ne);
+  for (int k = threadIdx.x; k < (q.ne + 1) / 2; k += DA_THREADS) {
+    const ff a = das_elem(q, g, 2 * k), b = das_elem(q, g, min(2 * k + 1, q.ne - 1));
+    xe_s[k] = make_ulonglong2(pack2(-a.hi, -b.hi), pack2(-a.lo, -b.lo));
+  }
+  int imin = 0x7FFFFFFF, imax = -0x7FFFFFFF;
   for (int t = 0; t < q.ntx; ++t) {
-    ut_s[t * DA_THREADS + threadIdx.x] = das_split(das_utx(q, g, x, z, t));
+    const float2 us = das_split(das_utx(q, g, x, z, t));
+    const int ui = __float_as_int(us.x);
+    imin = min(imin, ui);
+    imax = max(imax, ui);
+    ut_s[t * DA_THREADS + threadIdx.x] = us;
     s1_s[t * DA_THREADS + threadIdx.x] = 0.0f;
   }
-  float c0 = 0.0f, cp = 0.0f;  // sum slope u; sum slope du/dp
+  das_tx_range(imin, imax);
+  __syncthreads();
+  float c0 = 0.0f, cp = 0.0f;    // sum slope u; sum slope du/dp over the even elements
+  float c0b = 0.0f, cpb = 0.0f;  // and over the odd ones
+  const unsigned live = __ballot_sync(0xFFFFFFFFu, gp != 0.0f);
   if (gp != 0.0f) {
-    for (int e = 0; e < q.ne; ++e) {
-      const float2 ur = das_split(das_urx(das_rx(g, x, z), das_elem(q, g, e)));
-      float dwp;
-      const float w = apod_w(q, im, x.hi, z.hi, e, &dwp);
+    const DasRx2 rx = das_rx2(das_rx(g, x, z));
+    const bool dynamic = im.fnum > 0.0f;
+    auto element = [&](int e, float& w, float& dwp, float& drp) {
+      dwp = 0.0f;
+      w = dynamic ? apod_w(q, im, x.hi, z.hi, e, &dwp) : w_s[e];
       const float ce = (float)e - hn;
       const float dx = x.hi - ce * q.pitch;
-      const float drp = -dx * ce * kfs / sqrtf(fmaf(dx, dx, z.hi * z.hi));  // d(receive delay)/dp
-      for (int t = 0; t < q.ntx; ++t) {
-        int i;
-        float f;
-        das_tap(ut_s[t * DA_THREADS + threadIdx.x], ur, i, f);
-        const float* row = rf + ((size_t)t * q.ne + e) * q.ns;
-        const float a = (i >= 0 && i < q.ns) ? __ldg(&row[i]) : 0.0f;
-        const float b = (i + 1 >= 0 && i + 1 < q.ns) ? __ldg(&row[i + 1]) : 0.0f;
-        const float sl = w * (b - a);
-        s1_s[t * DA_THREADS + threadIdx.x] += sl;
-        c0 = fmaf(sl, (float)i + f, c0);
-        cp = fmaf(sl, fmaf(hn * fabsf(q.sin_tx[t]), kfs, drp), cp);
-        cp = fmaf(dwp, fmaf(f, b - a, a), cp);  // the weight's own pitch term (dynamic aperture)
+      drp = -dx * ce * kfs / sqrtf(fmaf(dx, dx, z.hi * z.hi));  // d(receive delay)/dp
+    };
+    auto tap = [&](auto inside, float2 u, float2 ur, const float* row, float w, float dwp, float drp, float dut,
+                   float& c, float& cpp) {
+      int i;
+      float f;
+      das_tap(u, ur, i, f);
+      float a, b;
+      if (inside) {
+        a = __ldg(&row[i]);
+        b = __ldg(&row[i + 1]);
+      } else {
+        a = (i >= 0 && i < q.ns) ? __ldg(&row[i]) : 0.0f;
+        b = (i + 1 >= 0 && i + 1 < q.ns) ? __ldg(&row[i + 1]) : 0.0f;
+      }
+      const float sl = w * (b - a);
+      c = fmaf(sl, (float)i + f, c);
+      cpp = fmaf(sl, fmaf(dut, kfs, drp), cpp);
+      if (dynamic) cpp = fmaf(dwp, fmaf(f, b - a, a), cpp);  // the weight's own pitch term
+      return sl;
+    };
+    const size_t tstride = (size_t)q.ne * q.ns;
+    for (int e = 0; e < q.ne; e += 2) {
+      const ulonglong2 xe = xe_s[e >> 1];
+      ff ua, ub;
+      das_urx2(rx, xe.x, xe.y, ua, ub);
+      const float2 ra = das_split(ua), rb = das_split(ub);
+      float wa, wb, da, db, pa, pb;
+      element(e, wa, da, pa);
+      const float* row = rf + (size_t)e * q.ns;
+      float2* u = ut_s + threadIdx.x;
+      float* s1 = s1_s + threadIdx.x;
+      auto pair = [&](auto inside) {
+        element(e + 1, wb, db, pb);
+#pragma unroll 2
+        for (int t = 0; t < q.ntx; ++t, row += tstride, u += DA_THREADS, s1 += DA_THREADS) {
+          const float2 ut = *u;
+          const float dut = hn * fabsf(q.sin_tx[t]);
+          const float sa = tap(inside, ut, ra, row, wa, da, pa, dut, c0, cp);
+          const float sb = tap(inside, ut, rb, row + q.ns, wb, db, pb, dut, c0b, cpb);
+          *s1 = (*s1 + sa) + sb;
+        }
+      };
+      if (e + 1 < q.ne) {
+        const bool in = das_inside(__float_as_int(ra.x), __float_as_int(rb.x), imin, imax, q.ns);
+        if (__all_sync(live, in)) pair(std::true_type());  // warp-uniform
+        else pair(std::false_type());
+      } else {
+        for (int t = 0; t < q.ntx; ++t, row += tstride, u += DA_THREADS, s1 += DA_THREADS)
+          *s1 += tap(std::false_type(), *u, ra, row, wa, da, pa, hn * fabsf(q.sin_tx[t]), c0, cp);
       }
     }
+    c0 += c0b;
+    cp += cpb;
   }
   float* out = part + (size_t)blockIdx.x * (2 + q.ntx);
   for (int t = 0; t < q.ntx; ++t) {
@@ -1267,9 +1331,11 @@ void launch_das(const Acq& q, const Img& im, const float* rf, float* irf, cudaSt
   const int tiles = ((im.nl + DAS_TL - 1) / DAS_TL) * ((im.nd + DAS_TD - 1) / DAS_TD);
   k_das<<<tiles, DAS_THREADS, das_smem(q.ne, q.ntx, im.fnum > 0.0f), st>>>(q, im, rf, irf);
 }
-int das_acq_blocks(const Img& im) { return (im.nl * im.nd + DA_THREADS - 1) / DA_THREADS; }
+int das_acq_blocks(const Img& im) {
+  return ((im.nl + DA_TL - 1) / DA_TL) * ((im.nd + DA_TD - 1) / DA_TD);
+}
 void launch_das_acq(const Acq& q, const Img& im, const float* rf, const float* gi, float* part, cudaStream_t st) {
-  k_das_acq<<<das_acq_blocks(im), DA_THREADS, das_acq_smem(q.ntx), st>>>(q, im, rf, gi, part);
+  k_das_acq<<<das_acq_blocks(im), DA_THREADS, das_acq_smem(q.ne, q.ntx), st>>>(q, im, rf, gi, part);
 }
 static std::atomic<int> g_das_adj_tiled{1};
 void launch_das_adj(const Acq& q, const Img& im, const float* gi, float* grf, int grid, cudaStream_t st,
@@ -1424,7 +1490,7 @@ cudaError_t image_set_attrs(int nd) {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_das_adj_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, DJ_SMEM_MAX);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_das_acq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)das_acq_smem(MAX_TX));
+  e = cudaFuncSetAttribute(k_das_acq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)das_acq_smem(MAX_ELEM, MAX_TX));
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_envelope, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(fft_line_bytes(nd) + sizeof(float2) * (size_t)(nd / 2)));
