@@ -1197,11 +1197,12 @@ __global__ void __launch_bounds__(256) k_envlog_vjp_fused(Img im, const float* _
 // derivative and the element weight are evaluated once per (pixel, element); the transmit delays
 // and the per-transmit sums S1 sit in shared memory in thread-major rows; the other two sums are
 // per-pixel scalars (their transmit weights are known before the sum).  Taps are checked against the
-// record once per pair of elements, for the whole warp: with a check per pixel, warps across the
-// record's end ran both loops.  Each block writes one row of 2 + ntx sums, reduced in a fixed order
-// (deterministic).  Bound by issue and by the gathers' latency.  128 elements, 11 transmits, 96 x
-// 512 pixels 377 -> 200 us; 95 elements, 6 transmits, 101 x 1024 pixels, a third of the taps past
-// the record 188 -> 157 us (170 with a check per pixel, 164 with one per tap).
+// record once per pair of elements and for the whole warp: a branch per pixel was slower even where
+// every tap lies inside (253 us against 200 in the first size below).  Each block writes one row of
+// 2 + ntx sums, reduced in a fixed order (deterministic).  Bound by issue and by the gathers'
+// latency.  128 elements, 11 transmits, 96 x 512 pixels 377 -> 200 us; 95 elements, 5 transmits,
+// F-number 1.5, 101 x 1024 pixels, 4 % of the taps past the record 188 -> 157 us (170 with a branch
+// per pixel, 164 with a check per tap).
 // ------------------------------------------------------------------------------------------
 constexpr int DA_THREADS = 256;
 constexpr int DA_TL = 8, DA_TD = 32;  // a block's lines x depths; a warp has 8 lines x 4 depths
