@@ -5,6 +5,7 @@
 #include <atomic>
 #include <cmath>
 #include <type_traits>
+#include <utility>
 
 #include <cooperative_groups.h>
 
@@ -985,12 +986,15 @@ __global__ void k_loss_partial(Img im, const float* __restrict__ b, const float*
 
 // The loss in one launch for images of at most LOSS_ONE pixels: one cluster of LOSS_CTAS blocks,
 // whose sums meet in the first one's shared memory (128 x 512 pixels: stage 11.6 us as two kernels,
-// 8.8 so; 256 x 1024: 13.4 and 12.1).
+// 8.8 so; 256 x 1024: 13.4 and 12.1).  A block's shared memory may be written from outside only once
+// the block has started: every block arrives at a cluster barrier as it begins and waits for the
+// others before its store, the pixels lying between the two.
 constexpr int LOSS_CTAS = 8, LOSS_THREADS = 1024, LOSS_ONE = 1 << 19;
 __global__ void __cluster_dims__(LOSS_CTAS, 1, 1) __launch_bounds__(LOSS_THREADS)
     k_loss_cluster(Img im, const float* __restrict__ b, const float* __restrict__ bref, float* gb, float* loss) {
   __shared__ float sums[LOSS_CTAS];
   cg::cluster_group cl = cg::this_cluster();
+  auto started = cl.barrier_arrive();
   const int n = im.nl * im.nd;
   const float inv = 1.0f / (float)n;
   float s = 0.0f;
@@ -1001,6 +1005,7 @@ __global__ void __cluster_dims__(LOSS_CTAS, 1, 1) __launch_bounds__(LOSS_THREADS
     if (gb) gb[i] = (im.l1 * (r > 0.0f ? 1.0f : (r < 0.0f ? -1.0f : 0.0f)) + 2.0f * im.l2 * r) * inv;
   }
   s = block_sum(s);
+  cl.barrier_wait(std::move(started));
   if (threadIdx.x == 0) cl.map_shared_rank(sums, 0)[cl.block_rank()] = s;
   cl.sync();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
