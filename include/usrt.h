@@ -173,14 +173,16 @@ enum {
   /* fault injection for tests of the timeout report (default 0): 1 makes the fused envelope
    * kernel's grid barrier wait for one arrival more than there are blocks, with a 1 ms limit,
    * so that the wait runs out: the image is written as NaN and us_get_status returns
-   * US_ERR_TIMEOUT.  The fault is injected from the host (a kernel argument); nothing faults. */
+   * US_ERR_TIMEOUT.  In the envelope's fused VJP every block but the first waits so: their lines
+   * come out as NaN, and the line of the image's maximum, which needs a sum over all of them, too.
+   * The fault is injected from the host (a kernel argument); nothing faults. */
   US_OPT_FAULT_BARRIER = 3,
   US_N_OPTS
 };
 int us_set_option(us_ctx* ctx, int option, int value);
 
-/* Status of the context's kernels outside the transport (TMA-staged DAS waits, the fused
- * envelope kernel's grid barrier): synchronises the device, then *device_status = US_OK, or
+/* Status of the context's kernels outside the transport (TMA-staged DAS waits, the grid barriers
+ * of the fused envelope kernel and of its VJP): synchronises the device, then *device_status = US_OK, or
  * US_ERR_TIMEOUT / US_ERR_OVERFLOW if any of them gave up since the last clear (their bounded
  * waits return instead of hanging).  clear != 0 resets the word.  The transport's own status
  * is reported by us_get_stats.  Returns US_ERR_ARG for a null argument, US_ERR_CUDA if the

@@ -1126,7 +1126,7 @@ int us_envlog_vjp(us_ctx* ctx, const us_img_desc* img, const float* irf_dev, con
   CKS(ws(ctx, W_SCAL, 4, st, &scal));
   StageScope sc_(ctx, US_STAGE_ENVLOG_VJP, 0, st);
   sc_.nk = launch_envlog_vjp(im, irf_dev, dL_dB_dev, env, key, part, np, scal, dL_dirf_dev, grid_of(ctx, 8), st,
-                             ctx->d_status);
+                             ctx->d_status, ctx->opts[US_OPT_FAULT_BARRIER]);
   CK(cudaGetLastError());
   return US_OK;
 }

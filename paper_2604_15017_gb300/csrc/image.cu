@@ -1078,12 +1078,16 @@ __global__ void k_envlog_vjp(Img im, const float* __restrict__ irf, const float*
 // memory, meets the others once for the maximum, and transforms back.  Only the line that holds
 // the maximum needs the sum S over all unclipped pixels: its block alone waits for the others'
 // partial sums (added in block order).  Both waits are bounded, as in k_envlog_fused; one that
-// expires makes the block's lines NaN and raises ST_TIMEOUT.  keyw: packed maximum, two arrival
-// counters (zeroed before the launch).  256 lines of 1024: 47 us as four kernels, which computed
-// the envelope's transform twice; 128 lines of 512: 30 us against 20.
+// expires makes the block's lines NaN and raises ST_TIMEOUT, and a block that went on without the
+// others' maximum gives NaN as its partial sum, so that the line with the maximum comes out NaN
+// too.  `extra` arrivals more than there are blocks (a test's injected fault, else 0) are awaited by
+// every block but block 0 in the first wait.  keyw: packed maximum, two arrival counters (zeroed
+// before the launch).  256 lines of 1024: 47 us as four kernels, which computed the envelope's
+// transform twice; 128 lines of 512: 30 us against 20.
 __global__ void __launch_bounds__(256) k_envlog_vjp_fused(Img im, const float* __restrict__ irf,
                                                           const float* __restrict__ gb, unsigned long long* keyw,
-                                                          float* part, float* gi, int* status, long long limit) {
+                                                          float* part, float* gi, int* status, int extra,
+                                                          long long limit) {
   extern __shared__ float2 sz[];
   const int N = im.nd, L = fft_slot(N) + 1;
   const int logN = 31 - __clz(N);
@@ -1116,10 +1120,11 @@ __global__ void __launch_bounds__(256) k_envlog_vjp_fused(Img im, const float* _
   }
   block_max_key(own, &best);
   __syncthreads();
-  auto wait = [&](unsigned long long* counter) {  // thread 0: until every block has arrived
+  // thread 0: until so many blocks have arrived
+  auto wait = [&](unsigned long long* counter, unsigned arrivals, long long cycles) {
     const long long t0 = clock64();
-    while (atomicAdd(counter, 0ull) < (unsigned long long)gridDim.x) {
-      if (clock64() - t0 > limit) {
+    while (atomicAdd(counter, 0ull) < (unsigned long long)arrivals) {
+      if (clock64() - t0 > cycles) {
         if (status) atomicOr(status, ST_TIMEOUT);
         s_ok = 0;
         break;
@@ -1132,7 +1137,7 @@ __global__ void __launch_bounds__(256) k_envlog_vjp_fused(Img im, const float* _
     atomicMax(&keyw[0], best);
     __threadfence();
     atomicAdd(&keyw[1], 1ull);
-    wait(&keyw[1]);
+    wait(&keyw[1], gridDim.x + (blockIdx.x ? (unsigned)extra : 0u), limit);
     best = atomicAdd(&keyw[0], 0ull);
   }
   __syncthreads();
@@ -1149,14 +1154,14 @@ __global__ void __launch_bounds__(256) k_envlog_vjp_fused(Img im, const float* _
     }
   sum = block_sum(sum);
   if (threadIdx.x == 0) {
-    part[blockIdx.x] = sum;
+    part[blockIdx.x] = s_ok ? sum : __int_as_float(0x7FC00000);
     __threadfence();
     atomicAdd(&keyw[2], 1ull);
   }
   const bool owner = emax > 0.0f && (am / N) % (int)gridDim.x == (int)blockIdx.x;
   float S = 0.0f;
   if (owner) {  // block-uniform
-    if (threadIdx.x == 0) wait(&keyw[2]);
+    if (threadIdx.x == 0) wait(&keyw[2], gridDim.x, 4 * limit);  // others may wait out the first before they arrive
     __syncthreads();
     float s = 0.0f;
     for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) s += __ldcg(&part[b]);
@@ -1456,7 +1461,8 @@ int launch_loss(const Img& im, const float* b, const float* bref, float* gb, flo
   return 2;
 }
 int launch_envlog_vjp(const Img& im, const float* irf, const float* gb, float* env, unsigned long long* key,
-                      float* part, int nparts, float* live_sum, float* gi, int grid, cudaStream_t st, int* status) {
+                      float* part, int nparts, float* live_sum, float* gi, int grid, cudaStream_t st, int* status,
+                      int fault_barrier) {
   if (g_envlog_fused.load() && gi != irf && gi != gb) {
     for (int lpb = 1; lpb <= 4; ++lpb) {  // lines per block: the fewest that keep the blocks co-resident
       const size_t smem = (lpb + 1) * fft_line_bytes(im.nd) + sizeof(float2) * (size_t)(im.nd / 2);
@@ -1465,9 +1471,10 @@ int launch_envlog_vjp(const Img& im, const float* irf, const float* gb, float* e
       // half of the resident blocks at most
       if (2 * nb > resident_blocks((const void*)k_envlog_vjp_fused, smem)) continue;
       if (cudaMemsetAsync(key, 0, 3 * sizeof(unsigned long long), st) != cudaSuccess) break;
-      long long limit = BARRIER_CYCLES;
+      int extra = fault_barrier ? 1 : 0;
+      long long limit = fault_barrier ? FAULT_BARRIER_CYCLES : BARRIER_CYCLES;
       void* args[] = {(void*)&im, (void*)&irf, (void*)&gb, (void*)&key, (void*)&part, (void*)&gi, (void*)&status,
-                      (void*)&limit};
+                      (void*)&extra, (void*)&limit};
       if (cudaLaunchCooperativeKernel((const void*)k_envlog_vjp_fused, dim3(nb), dim3(256), args, smem, st) == cudaSuccess)
         return 1;
       cudaGetLastError();  // the refused cooperative launch: fall back to the four kernels

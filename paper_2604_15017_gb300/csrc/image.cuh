@@ -29,7 +29,8 @@ int launch_envlog(const Img& im, const float* irf, float* env, unsigned long lon
 int launch_loss(const Img& im, const float* b, const float* bref, float* gb, float* part, int nparts, float* loss,
                 cudaStream_t st);
 int launch_envlog_vjp(const Img& im, const float* irf, const float* gb, float* env, unsigned long long* key,
-                      float* part, int nparts, float* live_sum, float* gi, int grid, cudaStream_t st, int* status);
+                      float* part, int nparts, float* live_sum, float* gi, int grid, cudaStream_t st, int* status,
+                      int fault_barrier = 0);
 cudaError_t image_set_attrs(int nd);
 
 }  // namespace usrt
