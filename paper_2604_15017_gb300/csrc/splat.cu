@@ -63,7 +63,8 @@ __global__ void k_pulse_table(SplatGeom g, float* G) {
 // Where the arrivals come from: the transport's packed list (its count on the device), or the
 // caller's four arrays, packed as they are read (a pass of its own that packed them, one atomic
 // per warp on one counter, took 200 us for 7.9M arrivals).  get() gives (row, tq, bits(a)), false
-// for an arrival outside the time range.
+// for an arrival outside the time range.  Up to 2^32 - 17 arrivals: the loops over them count in 64
+// bits, 32 would wrap before the end of such a list.
 struct PackedArrivals {
   const Arrival* arr;
   const uint32_t* n_arr;
@@ -105,9 +106,9 @@ __global__ void k_row_hist(Src src, uint32_t* row_cnt, int nrows) {
   if (blockIdx.x * blockDim.x >= n) return;
   for (int r = threadIdx.x; r < nrows; r += blockDim.x) h[r] = 0;
   __syncthreads();
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  for (size_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     uint32_t r;
-    if (src.row(i, r)) atomicAdd(&h[r], 1u);
+    if (src.row((uint32_t)i, r)) atomicAdd(&h[r], 1u);
   }
   __syncthreads();
   for (int r = threadIdx.x; r < nrows; r += blockDim.x)
@@ -171,17 +172,17 @@ __global__ void __launch_bounds__(SC_THREADS) k_row_scatter(Src src, const uint3
   uint32_t* h = sm;           // per-row count in this chunk
   uint32_t* base = sm + nrows;
   const uint32_t n = src.count();
-  for (uint32_t c0 = blockIdx.x * SC_CH; c0 < n; c0 += gridDim.x * SC_CH) {
+  for (size_t c0 = (size_t)blockIdx.x * SC_CH; c0 < n; c0 += (size_t)gridDim.x * SC_CH) {
     for (int r = threadIdx.x; r < nrows; r += blockDim.x) h[r] = 0;
     __syncthreads();
     uint32_t row[SC_PER], rank[SC_PER];
     uint2 val[SC_PER];
 #pragma unroll
     for (int k = 0; k < SC_PER; ++k) {
-      const uint32_t i = c0 + k * SC_THREADS + threadIdx.x;
+      const size_t i = c0 + k * SC_THREADS + threadIdx.x;
       row[k] = 0xFFFFFFFFu;
       uint32_t r;
-      if (i < n && src.get(i, r, val[k])) {
+      if (i < n && src.get((uint32_t)i, r, val[k])) {
         row[k] = r;
         rank[k] = atomicAdd(&h[r], 1u);
       }
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) k_row_splat(SplatGeom g, const
   __syncthreads();
   const uint32_t mask = (1u << TQ_FRAC) - 1u;
   // pass 1: histogram of bins
-  for (uint32_t i = a0 + tid; i < a1; i += ROW_THREADS) {
+  for (size_t i = (size_t)a0 + tid; i < a1; i += ROW_THREADS) {
     const int b = (int)(bucket[i].x >> TQ_FRAC) - TQ_OFFSET + HALO;
     if (b >= 0 && b < NB) atomicAdd(&hist[b], 1u);
   }
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) k_row_splat(SplatGeom g, const
   }
   __syncthreads();
   // pass 2: scatter into bin order (scratch shares the row's index range)
-  for (uint32_t i = a0 + tid; i < a1; i += ROW_THREADS) {
+  for (size_t i = (size_t)a0 + tid; i < a1; i += ROW_THREADS) {
     const uint2 v = bucket[i];
     const int b = (int)(v.x >> TQ_FRAC) - TQ_OFFSET + HALO;
     if (b >= 0 && b < NB) scratch[a0 + atomicAdd(&hist[b], 1u)] = v;
@@ -276,8 +277,8 @@ __global__ void __launch_bounds__(ROW_THREADS, 2) k_row_splat(SplatGeom g, const
     for (int i = tid; i < K_MOM * MS; i += ROW_THREADS) M[i] = 0.0f;
     __syncthreads();
     // segmented warp reduction of the moments over the bin-sorted arrivals
-    for (uint32_t base = r0 + (tid & ~31u); base < r1; base += ROW_THREADS) {
-      const uint32_t i = base + lane;
+    for (size_t base = (size_t)r0 + (tid & ~31u); base < r1; base += ROW_THREADS) {
+      const size_t i = base + lane;
       int b = -1;
       float m[K_MOM];
 #pragma unroll
