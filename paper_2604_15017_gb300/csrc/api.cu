@@ -408,9 +408,12 @@ struct Queues {
 // 1.0M 2.39 -> 2.25 ms, 1.4M 3.15 -> 2.78, 2.0M 3.73 -> 3.62, 3.1M 4.71 -> 4.97, 4.1M 5.77 -> 6.36;
 // 3 regions and 3000 scatterers, 2.0M 1.43 -> 1.26 ms, 4.1M 1.94 -> 1.93.
 constexpr uint32_t SMALL_PASS = 1u << 21;
-// scenes without scatterers and with at most this many triangles need no sort at any size (every
-// ray visits the same few nodes): two layers, 12 triangles, 6.4e5 paths 362 -> 268 us
-constexpr int UNSORTED_TRIS = 64;
+// Scenes without scatterers and with at most this many triangles leave the rays unsorted in larger
+// passes too (every ray visits the same few nodes).  Forward passes of 4M and of 16M paths, sorted
+// and unsorted, in us: two layers, 12 triangles, 844 and 739, 2781 and 2652; with boxes in them, 24
+// triangles 871 and 780, 2878 and 2793; 48 triangles 899 and 874, but 2965 and 3123; 60 triangles
+// 964 and 973, 3210 and 3557; 204 triangles 1180 and 1400, 4046 and 5269.
+constexpr int UNSORTED_TRIS = 24;
 
 int alloc_queues(us_ctx* ctx, long long n, cudaStream_t st, Queues& Q) {
   CKS(ws(ctx, W_QA_PA, n, st, &Q.a.pa));
