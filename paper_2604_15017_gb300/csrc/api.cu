@@ -475,7 +475,10 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
   A.sort = !(n <= SMALL_PASS || (sc->dev.n_scat == 0 && sc->dev.n_tris <= UNSORTED_TRIS));
   if (!A.sort) CKS(ws(ctx, W_QB_SURF, n, st, &Q.b.surf));
   NeeQ sorted = A.nee, unsorted;
-  const bool sort_jobs = any_jobs && A.sort;
+  // a large pass that leaves its rays unsorted sorts its secondary-ray jobs all the same when they are
+  // recorded for an adjoint, which reads them in their order: two rough layers, 8M paths, forward
+  // 2557 us unsorted and 2844 sorted, adjoint 2917 and 2394
+  const bool sort_jobs = any_jobs && (A.sort || (record && n > SMALL_PASS));
   if (sort_jobs) {
     CKS(ws(ctx, W_JOBU_JOB, jobs, st, &unsorted.job));
     CKS(ws(ctx, W_JOBU_JM, jobs, st, &unsorted.jm));
@@ -507,11 +510,11 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
   const bool side = do_nee && any_jobs && nee_pct > 0;
   Lane* L = ctx->L;
   if (side) CKS(ensure_side(ctx, L));
-  // unsorted rounds share no scratch: odd ones take another stream, so that a round's secondary rays
+  // rounds without a job sort share no scratch: odd ones take another stream, so that a round's secondary rays
   // need not wait for the previous round's (inverse-problem iteration 1017 -> 950 us, medium render
   // 1068 -> 1035); only for single calls: with the batch's lanes it made more streams than the
   // device has queues for (batch of 8 +3.5 %)
-  const bool two_sides = side && !A.sort && !L->stream;
+  const bool two_sides = side && !sort_jobs && !L->stream;
   const int nee_grid = side ? std::max(ctx->num_sms, grid_of(ctx, ctx->nee_per_sm) * nee_pct / 100)
                             : grid_of(ctx, ctx->nee_per_sm);
   RaySort rs;

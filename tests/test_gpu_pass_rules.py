@@ -25,10 +25,10 @@ def boxes(n, n_rays):
     return w
 
 
-def launches(ctx, w):
+def launches(ctx, w, **kw):
     sid = ctx.upload_workload(w)
     ctx.profile(True)
-    ctx.forward(sid, w["theta"], w["acq"], seed=3)
+    ctx.forward(sid, w["theta"], w["acq"], seed=3, **kw)
     torch.cuda.synchronize()
     n = {k: v[1] for k, v in ctx.profile_read().items()}
     ctx.profile(False)
@@ -47,3 +47,39 @@ def launches(ctx, w):
 ])
 def test_rays_are_sorted_in_large_passes_of_scenes_with_many_nodes(ctx, make, rays):
     assert (launches(ctx, make())["ray_sort"] > 0) == rays
+
+
+@pytest.mark.parametrize("make,jobs,recorded", [
+    (lambda: P.with_roughness(boxes(0, 32768), [0.0, 0.3]), False, False),
+    (lambda: P.with_roughness(boxes(0, LARGE), [0.0, 0.3]), False, True),  # its rays are not sorted
+    (lambda: P.with_roughness(boxes(2, LARGE), [0.0, 0.3]), True, True),
+    (lambda: boxes(0, LARGE), False, False),                               # none to sort
+    (lambda: P.slab_scatterers(n_rays=32768, n_scat=500, k_max=2), False, False),
+    (lambda: P.slab_scatterers(n_rays=LARGE, n_scat=500, k_max=2), True, True),
+])
+def test_secondary_ray_jobs_are_sorted_in_large_passes(ctx, make, jobs, recorded):
+    w = make()
+    assert (launches(ctx, w)["job_sort"] > 0) == jobs
+    assert (launches(ctx, w, keep_record=True)["job_sort"] > 0) == recorded
+
+
+@pytest.mark.parametrize("rough_nee", [0, 1])
+def test_recorded_rough_jobs_in_a_large_unsorted_pass(ctx, rough_nee):
+    """Two rough layers at more than 2^21 paths (unsorted rays, sorted jobs when recorded): channel data and
+    gradient equal the sum over four sub-apertures, whose small passes sort nothing, for one
+    dL/dRF, up to the FP32 order of sums (as in test_gpu_edges.py)."""
+    w = P.with_roughness(boxes(0, LARGE), [0.0, 0.3])
+    acq = dict(w["acq"], rough_nee=rough_nee)
+    sid = ctx.upload_workload(w)
+    rf, _ = ctx.forward(sid, w["theta"], acq, seed=3, keep_record=True)
+    grf = torch.randn(rf.shape, generator=torch.Generator("cuda").manual_seed(1), device="cuda")
+    g = ctx.transport_vjp(sid, w["theta"], acq, 3, grf)
+    rf_sum, g_sum = torch.zeros_like(rf), torch.zeros_like(g)
+    for b in range(4):
+        part = dict(acq, tx_elem=16 * b, n_tx_elem=16)
+        rf_sum += ctx.forward(sid, w["theta"], part, seed=3, keep_record=True)[0]
+        g_sum += ctx.transport_vjp(sid, w["theta"], part, 3, grf)
+    assert float(rf.norm()) > 0 and float(g.abs().max()) > 0
+    assert float((rf_sum - rf).norm()) <= 1e-5 * float(rf.norm())
+    assert torch.allclose(g_sum, g, rtol=1e-4, atol=1e-5 * float(g.abs().max())), (g, g_sum)
+    ctx.release_scene(sid)
