@@ -1464,12 +1464,15 @@ int launch_envlog_vjp(const Img& im, const float* irf, const float* gb, float* e
                       float* part, int nparts, float* live_sum, float* gi, int grid, cudaStream_t st, int* status,
                       int fault_barrier) {
   if (g_envlog_fused.load() && gi != irf && gi != gb) {
-    for (int lpb = 1; lpb <= 4; ++lpb) {  // lines per block: the fewest that keep the blocks co-resident
+    // lines per block: the fewest that keep the blocks co-resident, at most four (a block's lines follow
+    // one another).  One, two, three, four lines, four kernels, in us: 256 x 4096 75, 105, 152, 200, 112;
+    // 400 x 4096 -, -, 152, 200, 165; 600 x 4096 -, -, -, 201, 197; 608 x 2048 -, 68, 96, 102, 88;
+    // 1000 x 1024 -, -, -, 80, 92
+    for (int lpb = 1; lpb <= 4; ++lpb) {
       const size_t smem = (lpb + 1) * fft_line_bytes(im.nd) + sizeof(float2) * (size_t)(im.nd / 2);
       const int nb = (im.nl + lpb - 1) / lpb;
       if (smem > (size_t)FUSED_SMEM_MAX || nparts < nb) continue;
-      // half of the resident blocks at most
-      if (2 * nb > resident_blocks((const void*)k_envlog_vjp_fused, smem)) continue;
+      if (nb > resident_blocks((const void*)k_envlog_vjp_fused, smem)) continue;
       if (cudaMemsetAsync(key, 0, 3 * sizeof(unsigned long long), st) != cudaSuccess) break;
       int extra = fault_barrier ? 1 : 0;
       long long limit = fault_barrier ? FAULT_BARRIER_CYCLES : BARRIER_CYCLES;

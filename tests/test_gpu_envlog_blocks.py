@@ -1,0 +1,29 @@
+"""The envelope's VJP where its one launch goes from one line per block to two, three, four and to four
+kernels: by the number of lines (two blocks' partial sums per SM, 304) and, in long lines, by the
+blocks whose lines fit the SMs' shared memory together (304 of one line of 4096 depths, 152 of two or
+three, 760 of one of 2048).  Against the oracle, as in test_gpu_envlog.py."""
+import pytest
+import torch
+
+from test_gpu_edges import ctx  # noqa: F401  (the fixture)
+from test_gpu_envlog import image, test_envlog_vjp_one_launch_and_four as check
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("nl,nd", [(304, 16), (305, 16), (608, 64), (912, 64), (1216, 64), (1217, 64), (304, 4096),
+                                   (400, 4096), (608, 2048)])
+def test_lines_per_block(ctx, nl, nd):
+    check(ctx, nl, nd)
+
+
+@pytest.mark.parametrize("nl,nd,kernels", [(304, 16, 1), (1216, 64, 1), (1217, 64, 4), (304, 4096, 1), (608, 4096, 1),
+                                           (609, 4096, 4)])
+def test_launches(ctx, nl, nd, kernels):
+    irf = torch.randn(nl, nd, device="cuda")
+    ctx.profile(True)
+    ctx.envlog_vjp(image(nl, nd), irf, irf.clone())
+    torch.cuda.synchronize()
+    n = ctx.profile_read()["envlog_vjp"][1]
+    ctx.profile(False)
+    assert n == kernels
