@@ -27,3 +27,9 @@ def test_launches(ctx, nl, nd, kernels):
     n = ctx.profile_read()["envlog_vjp"][1]
     ctx.profile(False)
     assert n == kernels
+
+
+@pytest.mark.parametrize("nl,nd", [(1300, 16), (1217, 32), (1300, 64), (1217, 128), (1217, 256)])
+def test_short_lines_in_four_kernels(ctx, nl, nd):
+    # as many threads as a line has pixels, from 64 to 256
+    check(ctx, nl, nd)
