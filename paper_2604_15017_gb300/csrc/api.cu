@@ -99,7 +99,8 @@ struct us_ctx {
   std::vector<Lane*> lanes;
   Lane* L = nullptr;  // lane of the call in progress
   int num_sms = 148;
-  int trav_per_sm = 4;   // blocks per SM of the traversal grid
+  int trav_resident = 4;  // resident blocks per SM of the traversal
+  int trav_per_sm = 8;   // blocks per SM of its grid: by default two waves, a short tail without a long grid-stride loop
   int closest_per_sm = 4;  // resident blocks per SM of the joint closest-hit kernel
   int march_per_sm = 4;  // resident blocks per SM of the scatterer march
   int nee_per_sm = 4;    // resident blocks per SM of the secondary-ray kernel
@@ -565,7 +566,7 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
       if (A.joint) {
         launch_closest(A, grid_of(ctx, ctx->closest_per_sm), st);
       } else {
-        launch_traverse(A, grid_of(ctx, ctx->trav_per_sm), st);
+        launch_traverse(A, grid_of(ctx, ctx->trav_per_sm), ctx->trav_per_sm / ctx->trav_resident, st);
         if (scat) launch_march(A, grid_of(ctx, ctx->march_per_sm), st);
       }
     }
@@ -701,7 +702,8 @@ int us_create(us_ctx** out, int device, size_t mem_budget_bytes) {
   }
   ctx->opts[US_OPT_LANES] = 4;
   ctx->opts[US_OPT_NEE_STREAM] = 100;
-  ctx->trav_per_sm = traverse_blocks_per_sm();
+  ctx->trav_resident = traverse_blocks_per_sm();
+  ctx->trav_per_sm = 2 * ctx->trav_resident;
   ctx->march_per_sm = march_blocks_per_sm();
   ctx->closest_per_sm = closest_blocks_per_sm();
   ctx->nee_per_sm = nee_blocks_per_sm();
@@ -1526,9 +1528,8 @@ int us_autotune_batch(us_ctx* ctx, int n, const us_request* reqs, void* stream, 
                       int* best_trav_per_sm) {
   if (!ctx || n < 1 || !reqs) return fail(ctx, US_ERR_ARG, "invalid batch");
   cudaStream_t st = (cudaStream_t)stream;
-  const int base_trav = traverse_blocks_per_sm() / 2;  // resident blocks of the traversal kernel
   const int lane_opts[] = {1, 2, 4, 8};
-  const int trav_opts[] = {1, 2, 4};
+  const int trav_opts[] = {ctx->trav_resident, 2 * ctx->trav_resident, 4 * ctx->trav_resident};
   float best = 3.0e38f;
   int bl = ctx->opts[US_OPT_LANES], bt = ctx->trav_per_sm;
   cudaEvent_t e0, e1;
@@ -1537,7 +1538,7 @@ int us_autotune_batch(us_ctx* ctx, int n, const us_request* reqs, void* stream, 
   for (int lo : lane_opts)
     for (int to : trav_opts) {
       ctx->opts[US_OPT_LANES] = lo;
-      ctx->trav_per_sm = base_trav * to;
+      ctx->trav_per_sm = to;
       CKS(us_forward_batch(ctx, n, reqs, stream));  // warm-up: grows the lanes' workspaces
       CK(cudaEventRecord(e0, st));
       CKS(us_forward_batch(ctx, n, reqs, stream));

@@ -168,8 +168,8 @@ __device__ __forceinline__ void traverse_rays(const TransportArgs& A, uint32_t b
   }
   if (overflow) atomicOr(&A.cnt->status, ST_OVERFLOW);
 }
-__global__ void __launch_bounds__(TRAV_THREADS, 8) k_traverse(TransportArgs A) {
-  traverse_rays(A, blockIdx.x, gridDim.x, 2u);
+__global__ void __launch_bounds__(TRAV_THREADS, 8) k_traverse(TransportArgs A, uint32_t waves) {
+  traverse_rays(A, blockIdx.x, gridDim.x, waves);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1033,7 +1033,9 @@ void launch_generate(const TransportArgs& a, long long path0, uint32_t n, const 
 void launch_generate_unsorted(const TransportArgs& a, long long path0, uint32_t n, int grid, cudaStream_t st) {
   k_generate<<<min((uint32_t)grid, (n + 255u) / 256u), 256, 0, st>>>(a, path0, n);
 }
-void launch_traverse(const TransportArgs& a, int grid, cudaStream_t st) { k_traverse<<<grid, TRAV_THREADS, 0, st>>>(a); }
+void launch_traverse(const TransportArgs& a, int grid, int waves, cudaStream_t st) {
+  k_traverse<<<grid, TRAV_THREADS, 0, st>>>(a, (uint32_t)waves);
+}
 void launch_march(const TransportArgs& a, int grid, cudaStream_t st) { k_march<<<grid, MARCH_THREADS, 0, st>>>(a); }
 void launch_closest(const TransportArgs& a, int grid, cudaStream_t st) { k_closest<<<grid, TRAV_THREADS, 0, st>>>(a); }
 int closest_blocks_per_sm() {
@@ -1049,7 +1051,7 @@ int march_blocks_per_sm() {
 int traverse_blocks_per_sm() {
   int b = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_traverse, TRAV_THREADS, 0) != cudaSuccess || b < 1) b = 4;
-  return 2 * b;  // two waves of resident blocks: a short tail without a long grid-stride loop
+  return b;
 }
 void launch_interact(const TransportArgs& a, int grid, cudaStream_t st) { k_interact<<<grid, IA_THREADS, 0, st>>>(a); }
 void launch_nee(const TransportArgs& a, int grid, cudaStream_t st) { k_nee<<<grid, NEE_THREADS, 0, st>>>(a); }

@@ -122,8 +122,8 @@ void launch_generate(const TransportArgs& a, long long path0, uint32_t n, const 
 // emission in path order, for a pass without the coherence sort
 void launch_generate_unsorted(const TransportArgs& a, long long path0, uint32_t n, int grid, cudaStream_t st);
 constexpr int TRAV_THREADS = 128;
-void launch_traverse(const TransportArgs& a, int grid, cudaStream_t st);
-int traverse_blocks_per_sm();  // blocks per SM of the traversal grid
+void launch_traverse(const TransportArgs& a, int grid, int waves, cudaStream_t st);  // waves of resident blocks in grid
+int traverse_blocks_per_sm();  // resident blocks per SM of the traversal
 constexpr int MARCH_THREADS = 128;
 void launch_march(const TransportArgs& a, int grid, cudaStream_t st);
 static_assert(MARCH_THREADS == TRAV_THREADS, "k_closest's blocks do either");
