@@ -494,7 +494,10 @@ typedef struct {
 int us_forward_batch(us_ctx* ctx, int n, const us_request* reqs, void* stream);
 
 /* Autotuner: times the batch for lane counts {1, 2, 4, 8} and traversal grids of {1, 2, 4} x
- * the resident blocks per SM, keeps the fastest on the context and reports it.  Synchronous. */
+ * the resident blocks per SM, keeps the fastest on the context and reports it.  The grids only
+ * where some request has a traversal launch of its own (no scatterers, or more than 2^21 paths:
+ * smaller passes search surfaces and scatterers in one launch, on a grid that is not tuned); else
+ * the context's grid stays and is reported.  Synchronous. */
 int us_autotune_batch(us_ctx* ctx, int n, const us_request* reqs, void* stream, int* best_lanes,
                       int* best_trav_per_sm);
 

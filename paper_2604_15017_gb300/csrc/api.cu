@@ -415,6 +415,8 @@ constexpr uint32_t SMALL_PASS = 1u << 21;
 // triangles 871 and 780, 2878 and 2793; 48 triangles 899 and 874, but 2965 and 3123; 60 triangles
 // 964 and 973, 3210 and 3557; 204 triangles 1180 and 1400, 4046 and 5269.
 constexpr int UNSORTED_TRIS = 24;
+// whether a pass searches surfaces and scatterers in one launch (else k_traverse, then k_march)
+bool joint_search(const SceneGPU* sc, long long n_paths) { return sc->dev.n_scat > 0 && n_paths <= SMALL_PASS; }
 
 int alloc_queues(us_ctx* ctx, long long n, cudaStream_t st, Queues& Q) {
   CKS(ws(ctx, W_QA_PA, n, st, &Q.a.pa));
@@ -561,7 +563,7 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
     if (sort_jobs) A.nee = unsorted;
     {
       const bool scat = sc->dev.n_scat > 0;
-      A.joint = scat && n <= SMALL_PASS;
+      A.joint = joint_search(sc, n);
       StageScope sc_(ctx, US_STAGE_TRAVERSE, scat && !A.joint ? 2 : 1, st);
       if (A.joint) {
         launch_closest(A, grid_of(ctx, ctx->closest_per_sm), st);
@@ -1529,7 +1531,18 @@ int us_autotune_batch(us_ctx* ctx, int n, const us_request* reqs, void* stream, 
   if (!ctx || n < 1 || !reqs) return fail(ctx, US_ERR_ARG, "invalid batch");
   cudaStream_t st = (cudaStream_t)stream;
   const int lane_opts[] = {1, 2, 4, 8};
-  const int trav_opts[] = {ctx->trav_resident, 2 * ctx->trav_resident, 4 * ctx->trav_resident};
+  // the traversal's grid is tried where a request has such a launch; else every grid would be the same
+  // batch, and noise would choose the one that later passes of the context get
+  std::vector<int> trav_opts = {ctx->trav_per_sm};
+  for (int j = 0; j < n; ++j) {
+    const auto sc = ctx->scenes.find(reqs[j].scene);
+    Acq q;
+    if (sc == ctx->scenes.end() || make_acq(ctx, reqs[j].acq, 0, q) != US_OK) continue;  // the batch reports it
+    if (!joint_search(&sc->second, q.rays_per_tx * q.ntx)) {
+      trav_opts = {ctx->trav_resident, 2 * ctx->trav_resident, 4 * ctx->trav_resident};
+      break;
+    }
+  }
   float best = 3.0e38f;
   int bl = ctx->opts[US_OPT_LANES], bt = ctx->trav_per_sm;
   cudaEvent_t e0, e1;

@@ -1,4 +1,5 @@
-"""What the batch autotuner chooses, and what its choices leave alone."""
+"""What the batch autotuner may choose: a traversal grid only where a request of the batch launches the
+traversal by itself."""
 import pytest
 import torch
 
@@ -10,6 +11,19 @@ pytestmark = pytest.mark.gpu
 
 def item(ctx, w):
     return dict(scene=ctx.upload_workload(w), theta=w["theta"], acq=w["acq"], img=w["img"], seed=1)
+
+
+def test_traversal_grid_is_tuned_only_where_it_is_used():
+    ctx = usrt.Context(0)
+    joint = usrt.Batch(ctx, [item(ctx, P.slab_scatterers(n_rays=100, n_scat=500)) for _ in range(2)])
+    grids = {joint.autotune()[1] for _ in range(6)}
+    assert len(grids) == 1  # nothing in this batch depends on it
+    grid = grids.pop()
+    for w in (P.two_layer(n_rays=100), P.slab_scatterers(n_rays=33000, n_scat=500)):
+        lanes, tuned = usrt.Batch(ctx, [item(ctx, w)]).autotune()
+        assert lanes in (1, 2, 4, 8) and tuned in (grid // 2, grid, 2 * grid)
+        assert joint.autotune()[1] == tuned  # and stays what was tuned
+    ctx.close()
 
 
 @pytest.mark.parametrize("n_rays", [1, 40, 3000])
