@@ -206,13 +206,13 @@ __global__ void __launch_bounds__(TRAV_THREADS, 8) k_traverse(TransportArgs A, u
 constexpr int MARCH_CHUNK = 32;
 constexpr int MARCH_REFILL_MIN = 8;
 
-// block `block` of `blocks` resident ones.  JOINT: rays before `unbounded`, whose surface hit is not
-// known yet, are searched to the end of the grid, and every ray's scat is written (t = 3e38:
-// none).  Else every ray is searched to its surface hit, and one that meets a scatterer first
-// gets its scat written and the flag set in its hit's code (writing every scat cost 2 % of the
-// march in the inclusion frame).
+// block `block` of `blocks` resident ones.  JOINT (an unsorted queue, whose surfaces are searched at
+// the same time): a ray that does not carry its surface hit is searched to the end of the grid, and
+// every ray's scat is written (t = 3e38: none).  Else every ray is searched to its surface hit, and
+// one that meets a scatterer first gets its scat written and the flag set in its hit's code (writing
+// every scat cost 2 % of the march in the inclusion frame).
 template <bool JOINT>
-__device__ __forceinline__ void march_rays(const TransportArgs& A, uint32_t block, uint32_t blocks, uint32_t unbounded) {
+__device__ __forceinline__ void march_rays(const TransportArgs& A, uint32_t block, uint32_t blocks) {
   const SceneDev& S = A.S;
   const uint32_t n = A.cnt->live[A.k];
   uint32_t* claim = &A.cnt->march[A.k];
@@ -271,11 +271,11 @@ __device__ __forceinline__ void march_rays(const TransportArgs& A, uint32_t bloc
         const float4 wt = A.qin.wt[ray];
         const float3 o = xyz(pa), w = xyz(wt);
         r2 = ray2(o, w);
-        if (JOINT && !A.sort) {
+        if (JOINT) {
           tbest = A.qin.surf[ray].x;  // carried, or none
           if (tbest < 0.0f) tbest = 3.0e38f;
         } else {
-          tbest = JOINT && ray < unbounded ? 3.0e38f : A.hits[ray].x;
+          tbest = A.hits[ray].x;
         }
         prev = A.qin.meta[ray].y;
         cbest = NO_SCAT;
@@ -365,19 +365,20 @@ __device__ __forceinline__ void march_rays(const TransportArgs& A, uint32_t bloc
 }
 
 __global__ void __launch_bounds__(MARCH_THREADS, 7) k_march(TransportArgs A) {
-  if (A.cnt->live[A.k] > 0u) march_rays<false>(A, blockIdx.x, gridDim.x, 0u);
+  if (A.cnt->live[A.k] > 0u) march_rays<false>(A, blockIdx.x, gridDim.x);
 }
 
-// Both searches of a round, side by side, for passes that do not keep the GPU full: the first half of the (resident)
-// blocks walk the BVH, the second half march the grid, without the surface bound for the rays
-// whose surface hit is not known yet.  Such a round lasts as long as the longest chain of
-// either search, so what the missing bound adds does not show, and the two chains overlap.
+// Both searches of a round, side by side, for passes that do not keep the GPU full (their queues are
+// not sorted): the first half of the (resident) blocks walk the BVH, the second half march the grid,
+// without the surface bound for the rays whose surface hit is not known yet.  Such a round lasts as
+// long as the longest chain of either search, so what the missing bound adds does not show, and the
+// two chains overlap.
 __global__ void __launch_bounds__(TRAV_THREADS, 7) k_closest(TransportArgs A) {
   const uint32_t half = gridDim.x / 2;
   if (blockIdx.x < half)
     traverse_rays(A, blockIdx.x, half, 1u);
   else if (A.cnt->live[A.k] > 0u)
-    march_rays<true>(A, blockIdx.x - half, gridDim.x - half, A.sort ? *A.trav_n : 0u);
+    march_rays<true>(A, blockIdx.x - half, gridDim.x - half);
 }
 
 // ------------------------------------------------------------------------------------------
