@@ -202,8 +202,12 @@ __global__ void __launch_bounds__(TRAV_THREADS, 8) k_traverse(TransportArgs A, u
 // rays: 1424 us, 790, 680, with the joint launch 408, now 375.
 // ------------------------------------------------------------------------------------------
 // 32-ray claims and a refill at 8 idle lanes, measured against 64 and 128 rays, 4, 6, 12 and 16 lanes
-// (inclusion frame 23.0 ms with 4 lanes, 22.7 with 6, 22.5 with 8)
+// (inclusion frame 23.0 ms with 4 lanes, 22.7 with 6, 22.5 with 8).  Rounds of more than MARCH_MANY
+// rays claim 64 at a time: where most rays pass the spheres by, the claims queue up at their one
+// counter (16M paths, 1000 spheres: forward 4.10 ms with 32, 3.83 with 64; inclusion frame 16.47 and
+// 16.47; but 3.5M paths, 30,000 spheres 2.61 and 2.63)
 constexpr int MARCH_CHUNK = 32;
+constexpr uint32_t MARCH_MANY = 1u << 22;
 constexpr int MARCH_REFILL_MIN = 8;
 
 // block `block` of `blocks` resident ones.  JOINT (an unsorted queue, whose surfaces are searched at
@@ -221,7 +225,7 @@ __device__ __forceinline__ void march_rays(const TransportArgs& A, uint32_t bloc
   const uint32_t warps = blocks * (MARCH_THREADS / 32);
   const uint32_t lanes = warp_lanes(n, warps);
   const uint32_t lane_mask = lanes >= 32u ? 0xFFFFFFFFu : (1u << lanes) - 1u;
-  const uint32_t chunk = lanes >= 32u ? (uint32_t)MARCH_CHUNK : lanes;
+  const uint32_t chunk = lanes < 32u ? lanes : (uint32_t)(n > MARCH_MANY ? 2 * MARCH_CHUNK : MARCH_CHUNK);
   const int refill_min = min(MARCH_REFILL_MIN, (int)lanes);
   const float h = S.gh;
   const int nx = S.gnx, ny = S.gny, nz = S.gnz;

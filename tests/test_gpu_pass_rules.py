@@ -83,3 +83,19 @@ def test_recorded_rough_jobs_in_a_large_unsorted_pass(ctx, rough_nee):
     assert float((rf_sum - rf).norm()) <= 1e-5 * float(rf.norm())
     assert torch.allclose(g_sum, g, rtol=1e-4, atol=1e-5 * float(g.abs().max())), (g, g_sum)
     ctx.release_scene(sid)
+
+
+def test_a_march_of_more_rays_makes_the_same_records(ctx):
+    """More than 2^22 rays are claimed 64 at a time: word for word the records of sub-apertures of at most
+    2^21 paths, which claim fewer and are not sorted."""
+    w = P.slab_scatterers(n_rays=66000, n_scat=2000, k_max=2)
+    acq = w["acq"]
+    assert acq["n_elem"] * acq["n_rays"] > 1 << 22
+    sid = ctx.upload_workload(w)
+    ctx.forward(sid, w["theta"], acq, seed=5, keep_record=True)
+    full = ctx.record(0, acq["n_elem"] * acq["n_rays"], acq["k_max"]).clone()
+    m = 16 * acq["n_rays"]
+    for b in range(4):
+        ctx.forward(sid, w["theta"], dict(acq, tx_elem=16 * b, n_tx_elem=16), seed=5, keep_record=True)
+        assert torch.equal(ctx.record(0, m, acq["k_max"]), full[b * m:(b + 1) * m])
+    ctx.release_scene(sid)
