@@ -985,11 +985,14 @@ __global__ void k_loss_partial(Img im, const float* __restrict__ b, const float*
 }
 
 // The loss in one launch for images of at most LOSS_ONE pixels: one cluster of LOSS_CTAS blocks,
-// whose sums meet in the first one's shared memory (128 x 512 pixels: stage 11.6 us as two kernels,
-// 8.8 so; 256 x 1024: 13.4 and 12.1).  A block's shared memory may be written from outside only once
-// the block has started: every block arrives at a cluster barrier as it begins and waits for the
-// others before its store, the pixels lying between the two.
-constexpr int LOSS_CTAS = 8, LOSS_THREADS = 1024, LOSS_ONE = 1 << 19;
+// whose sums meet in the first one's shared memory.  A block's shared memory may be written from
+// outside only once the block has started: every block arrives at a cluster barrier as it begins and
+// waits for the others before its store, the pixels lying between the two.
+// Bound by the reads of eight SMs.  In a graph, two kernels and one, in us: 128 x 512 pixels 3.3 and
+// 3.2, 256 x 1024 3.9 and 5.4, 512 x 1024 4.5 and 8.7; but each launch costs the host 3 us as well, and
+// envelope, loss and VJP called after one another take 37.2 and 32.3 us, 53.2 and 52.4, at 256 x 2048
+// 70.9 and 72.8: one launch up to 2^18 pixels.
+constexpr int LOSS_CTAS = 8, LOSS_THREADS = 1024, LOSS_ONE = 1 << 18;
 __global__ void __cluster_dims__(LOSS_CTAS, 1, 1) __launch_bounds__(LOSS_THREADS)
     k_loss_cluster(Img im, const float* __restrict__ b, const float* __restrict__ bref, float* gb, float* loss) {
   __shared__ float sums[LOSS_CTAS];

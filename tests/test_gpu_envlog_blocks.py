@@ -33,3 +33,21 @@ def test_launches(ctx, nl, nd, kernels):
 def test_short_lines_in_four_kernels(ctx, nl, nd):
     # as many threads as a line has pixels, from 64 to 256
     check(ctx, nl, nd)
+
+
+@pytest.mark.parametrize("nl,kernels", [(256, 1), (257, 2)])
+def test_loss_launches(ctx, nl, kernels):
+    # one launch up to 2^18 pixels; the values at both sides against 64 bits
+    b, ref = (-60.0 * torch.rand(nl, 1024, generator=torch.Generator().manual_seed(k)).cuda() for k in (1, 2))
+    img = dict(image(nl, 1024), lambda1=0.5, lambda2=0.25)
+    ctx.profile(True)
+    loss, gb = ctx.loss(img, b, ref)
+    torch.cuda.synchronize()
+    n = ctx.profile_read()["loss"][1]
+    ctx.profile(False)
+    assert n == kernels
+    r = b.double() - ref.double()
+    want = float((0.5 * r.abs() + 0.25 * r * r).mean())
+    assert abs(float(loss) - want) <= 1e-5 * want  # positive terms in chains of up to 100
+    g = (0.5 * r.sign() + 0.5 * r) / r.numel()
+    assert float((gb - g).abs().max()) <= 1e-6 * float(g.abs().max())
