@@ -568,7 +568,7 @@ int run_transport(us_ctx* ctx, const SceneGPU* sc, const Media& med, const Acq& 
       if (A.joint) {
         launch_closest(A, grid_of(ctx, ctx->closest_per_sm), st);
       } else {
-        launch_traverse(A, grid_of(ctx, ctx->trav_per_sm), ctx->trav_per_sm / ctx->trav_resident, st);
+        launch_traverse(A, grid_of(ctx, ctx->trav_per_sm), grid_of(ctx, ctx->trav_resident), st);
         if (scat) launch_march(A, grid_of(ctx, ctx->march_per_sm), st);
       }
     }

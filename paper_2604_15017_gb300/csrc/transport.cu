@@ -136,15 +136,15 @@ __device__ __forceinline__ uint32_t warp_lanes(uint32_t n, uint32_t warps) {
 // of the BVH are fetched once per warp.  The scatterers are searched next by k_march below the
 // distance written here.
 // ------------------------------------------------------------------------------------------
-// block `block` of `blocks` (`waves` waves of resident blocks)
-__device__ __forceinline__ void traverse_rays(const TransportArgs& A, uint32_t block, uint32_t blocks, uint32_t waves) {
+// block `block` of `blocks`, of which `warps` warps run at a time
+__device__ __forceinline__ void traverse_rays(const TransportArgs& A, uint32_t block, uint32_t blocks, uint32_t warps) {
   if (block == 0 && threadIdx.x == 0)  // secondary jobs of this round follow the previous rounds'
     A.cnt->nee_off[A.k] = A.k ? A.cnt->nee_off[A.k - 1] + A.cnt->nee[A.k - 1] : 0u;
   // in a sorted queue the rays that carry their surface hit come last (and their hits are there)
   const uint32_t n = A.sort ? *A.trav_n : A.cnt->live[A.k];
   // one wave of warps takes a small queue a few lanes each (warp_lanes); a larger one is walked
   // grid-stride, consecutive rays in one block
-  const uint32_t lanes = warp_lanes(n, blocks * (TRAV_THREADS / 32) / waves);
+  const uint32_t lanes = warp_lanes(n, warps);
   const uint32_t lane = threadIdx.x & 31u;
   const bool spread = lanes < 32u;
   uint32_t i = block * TRAV_THREADS + threadIdx.x;
@@ -168,8 +168,8 @@ __device__ __forceinline__ void traverse_rays(const TransportArgs& A, uint32_t b
   }
   if (overflow) atomicOr(&A.cnt->status, ST_OVERFLOW);
 }
-__global__ void __launch_bounds__(TRAV_THREADS, 8) k_traverse(TransportArgs A, uint32_t waves) {
-  traverse_rays(A, blockIdx.x, gridDim.x, waves);
+__global__ void __launch_bounds__(TRAV_THREADS, 8) k_traverse(TransportArgs A, uint32_t warps) {
+  traverse_rays(A, blockIdx.x, gridDim.x, warps);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(MARCH_THREADS, 7) k_march(TransportArgs A) {
 __global__ void __launch_bounds__(TRAV_THREADS, 7) k_closest(TransportArgs A) {
   const uint32_t half = gridDim.x / 2;
   if (blockIdx.x < half)
-    traverse_rays(A, blockIdx.x, half, 1u);
+    traverse_rays(A, blockIdx.x, half, half * (TRAV_THREADS / 32));
   else if (A.cnt->live[A.k] > 0u)
     march_rays<true>(A, blockIdx.x - half, gridDim.x - half);
 }
@@ -1038,8 +1038,8 @@ void launch_generate(const TransportArgs& a, long long path0, uint32_t n, const 
 void launch_generate_unsorted(const TransportArgs& a, long long path0, uint32_t n, int grid, cudaStream_t st) {
   k_generate<<<min((uint32_t)grid, (n + 255u) / 256u), 256, 0, st>>>(a, path0, n);
 }
-void launch_traverse(const TransportArgs& a, int grid, int waves, cudaStream_t st) {
-  k_traverse<<<grid, TRAV_THREADS, 0, st>>>(a, (uint32_t)waves);
+void launch_traverse(const TransportArgs& a, int grid, int resident, cudaStream_t st) {
+  k_traverse<<<grid, TRAV_THREADS, 0, st>>>(a, (uint32_t)resident * (TRAV_THREADS / 32));
 }
 void launch_march(const TransportArgs& a, int grid, cudaStream_t st) { k_march<<<grid, MARCH_THREADS, 0, st>>>(a); }
 void launch_closest(const TransportArgs& a, int grid, cudaStream_t st) { k_closest<<<grid, TRAV_THREADS, 0, st>>>(a); }

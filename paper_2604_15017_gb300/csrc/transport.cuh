@@ -122,7 +122,7 @@ void launch_generate(const TransportArgs& a, long long path0, uint32_t n, const 
 // emission in path order, for a pass without the coherence sort
 void launch_generate_unsorted(const TransportArgs& a, long long path0, uint32_t n, int grid, cudaStream_t st);
 constexpr int TRAV_THREADS = 128;
-void launch_traverse(const TransportArgs& a, int grid, int waves, cudaStream_t st);  // waves of resident blocks in grid
+void launch_traverse(const TransportArgs& a, int grid, int resident, cudaStream_t st);  // resident of its blocks at a time
 int traverse_blocks_per_sm();  // resident blocks per SM of the traversal
 constexpr int MARCH_THREADS = 128;
 void launch_march(const TransportArgs& a, int grid, cudaStream_t st);
