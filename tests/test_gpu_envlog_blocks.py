@@ -51,3 +51,28 @@ def test_loss_launches(ctx, nl, kernels):
     assert abs(float(loss) - want) <= 1e-5 * want  # positive terms in chains of up to 100
     g = (0.5 * r.sign() + 0.5 * r) / r.numel()
     assert float((gb - g).abs().max()) <= 1e-6 * float(g.abs().max())
+
+
+def test_two_launches_that_each_fill_the_gpu(ctx):
+    """304 lines of 4096 depths take every block that fits; two such VJPs on two streams, beside each other,
+    wait for blocks of their own launch only and give the bits of one after the other."""
+    from paper_2604_15017_gb300 import usrt
+
+    other = usrt.Context(0)
+    img = image(304, 4096)
+    sides = []
+    for c, k in ((ctx, 1), (other, 2)):
+        gen = torch.Generator("cuda").manual_seed(k)
+        irf, gb = (torch.randn(304, 4096, generator=gen, device="cuda") for _ in range(2))
+        sides.append((c, irf, gb, torch.cuda.Stream(), c.envlog_vjp(img, irf, gb)))
+    torch.cuda.synchronize()
+    out = [[], []]
+    for _ in range(20):
+        for j, (c, irf, gb, st, _) in enumerate(sides):
+            with torch.cuda.stream(st):
+                out[j].append(c.envlog_vjp(img, irf, gb))
+    torch.cuda.synchronize()
+    for j, (c, *_, want) in enumerate(sides):
+        assert c.device_status() == usrt.US_OK
+        assert all(torch.equal(v, want) for v in out[j])
+    other.close()
