@@ -411,7 +411,9 @@ __device__ __forceinline__ void interact_one(const TransportArgs& A, uint32_t i,
   const Media& med = A.med;
   const int K1 = q.kmax + 1;
   float2 ks = A.hits[i];  // the surface hit
-  const float2 sc = A.scat[i];  // read with the slot's other words; what it holds counts below
+  // read with the slot's other words; it counts (below) only where a scatterer was met, and is never
+  // written otherwise except by the joint search
+  const float2 sc = A.scat[i];
   const uint32_t kc = __float_as_uint(ks.y);
   ks.y = __uint_as_float(kc & ~HIT_SCAT);
   float2 h = ks;  // or a scatterer before it
