@@ -386,7 +386,9 @@ int us_adjoint(us_ctx* ctx, uint64_t scene, const float* theta, const us_acq_des
  *   [2 + t] = dL/d(steering angle of transmit t) (per radian). */
 
 /* DAS part alone: sum_p dL/dI_rf(p) dI_rf(p)/d(c_bf, pitch, th_t) with the RF held fixed.  The slope
- * of each tap is that of the linear-interpolation interval holding its delay.  rf_dev: DEVICE
+ * of each tap is that of the linear-interpolation interval holding its delay.  dL/dpitch is NaN when
+ * a pixel with a nonzero gradient coincides with an element (z = 0, x = x_e): the receive distance
+ * has no derivative there.  rf_dev: DEVICE
  * float[n_tx][n_elem][n_samples]; dL_dirf_dev: DEVICE float[n_lines][n_depth].  Errors:
  * US_ERR_ARG (a null buffer, an invalid descriptor), US_ERR_OOM (workspace), US_ERR_CUDA. */
 int us_das_acq_vjp(us_ctx* ctx, const us_acq_desc* acq, const us_img_desc* img, const float* rf_dev,
